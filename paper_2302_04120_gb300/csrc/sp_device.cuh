@@ -18,11 +18,6 @@ __device__ __forceinline__ int wrap(int a, int n) { return a < 0 ? a + n : (a >=
 __device__ __forceinline__ int along(int side, int i, int j) { return side < 2 ? j : i; }
 __device__ __forceinline__ int side_len(const SpParams &P, int side) { return side < 2 ? P.ny : P.nx; }
 
-// Node (i, j) lies on side s (0: x = 0, 1: x = nx - 1, 2: y = 0, 3: y = ny - 1).
-__device__ __forceinline__ bool on_side(const SpParams &P, int s, int i, int j) {
-  return (s == 0 && i == 0) || (s == 1 && i == P.nx - 1) || (s == 2 && j == 0) || (s == 3 && j == P.ny - 1);
-}
-
 // Which side the link arriving at (i, j) along c = (cx, cy) comes through (source
 // node (i - cx, j - cy) outside the domain), or -1.  A link through a corner takes
 // the y-side, unless that y-side is a symmetry side (ysym: bit 0 for y = 0, bit 1
@@ -91,8 +86,62 @@ __device__ __forceinline__ void post_velocity(const SpParams &P, const S *src, i
     Fx += K<R>(P).bgx * dT;
     Fy += K<R>(P).bgy * dT;
   }
-  ux = (jx - (R)0.5 * K<R>(P).dt * Fx) / rho;
-  uy = (jy - (R)0.5 * K<R>(P).dt * Fy) / rho;
+  const R inv = (R)1 / rho;  // one division for both components
+  ux = (jx - (R)0.5 * K<R>(P).dt * Fx) * inv;
+  uy = (jy - (R)0.5 * K<R>(P).dt * Fy) * inv;
+}
+
+// ---- boundary links ---------------------------------------------------------
+// A link along (cx, cy) enters through the x-side cx > 0 ? 0 : 1 or the y-side cy > 0 ?
+// 2 : 3, known at compile time; in[s] says whether this node's links enter through side
+// s.  Every rule of Sec. 2.1 / 2.2 but the wet node is affine in one stored value:
+// f_q = +- raw + w_q (base + cu (lin + quad cu)), cu = c_q . u of the side.  So a node
+// gathers one value per link, then goes through the sides it lies on: forms a side's
+// coefficients and finishes that side's links.
+// The boundary frame is the critical path of a step on small and middle grids: its warps
+// run gather, coefficients and links one after the other with few warps beside them.
+// Selecting among four sides per link and per attribute took about 4000 instructions a
+// warp, whose fetch alone bounded the step (10 of 16 cycles per instruction waiting for
+// code).  Measured with the two forms, FP32, back-to-back steps: 2000 x 50 half channel,
+// D2Q9 + D2Q9, 13.6 -> 6.8 us; 2048 x 256 channel, D2Q9 + D2Q5, 12.9 -> 10.1 us (64 x 4
+// blocks); 128 x 32 channel 7.0 -> 3.7 us.
+struct NodeSides {
+  bool in[4];
+  int xm, xp;             // columns i - 1, i + 1 (wrapped)
+  long long r0, rm, rp;   // row offsets of j, j - 1, j + 1 (wrapped)
+};
+
+__device__ __forceinline__ NodeSides node_sides(const SpParams &P, int i, int j, int xper, int yper) {
+  NodeSides b;
+  b.in[0] = !xper && i == 0;
+  b.in[1] = !xper && i == P.nx - 1;
+  b.in[2] = !yper && j == 0;
+  b.in[3] = !yper && j == P.ny - 1;
+  b.xm = i == 0 ? P.nx - 1 : i - 1;
+  b.xp = i == P.nx - 1 ? 0 : i + 1;
+  b.r0 = (long long)j * P.pitch;
+  b.rm = (long long)(j == 0 ? P.ny - 1 : j - 1) * P.pitch;
+  b.rp = (long long)(j == P.ny - 1 ? 0 : j + 1) * P.pitch;
+  return b;
+}
+
+// Streaming source of a link along (cx, cy) within its plane.
+__device__ __forceinline__ long long stream_at(const NodeSides &b, int i, int cx, int cy) {
+  return (cy > 0 ? b.rm : cy < 0 ? b.rp : b.r0) + (cx > 0 ? b.xm : cx < 0 ? b.xp : i);
+}
+
+// Whether the link along (cx, cy) enters through side s: a corner link takes the y-side
+// unless that one is a symmetry plane (ysym bits) and the x-side stands.
+__host__ __device__ constexpr int side_x(int cx) { return cx > 0 ? 0 : 1; }
+__host__ __device__ constexpr int side_y(int cy) { return cy > 0 ? 2 : 3; }
+__host__ __device__ constexpr bool may_enter(int s, int cx, int cy) {
+  return s < 2 ? cx != 0 && side_x(cx) == s : cy != 0 && side_y(cy) == s;
+}
+template <bool SYM>
+__device__ __forceinline__ bool enters(const NodeSides &b, int s, int cx, int cy, int ysym) {
+  if (!may_enter(s, cx, cy) || !b.in[s]) return false;
+  if (s < 2) return cy == 0 || !b.in[side_y(cy)] || (SYM && ((ysym >> (side_y(cy) - 2)) & 1));
+  return !SYM || cx == 0 || !b.in[side_x(cx)] || !((ysym >> (s - 2)) & 1);
 }
 
 // Pull of all momentum populations at node (i, j), with boundary links.  SYM: the
@@ -111,83 +160,58 @@ __device__ __forceinline__ void pull_f(const SpParams &P, const S *src, int i, i
     for (int q = 0; q < 9; q++) f[q] = (R)src[q * P.plane + n];
     return;
   }
-  const R c = K<R>(P).c, inv_cs2 = K<R>(P).inv_cs2;
   // 1. gather, branch-free so that all nine loads are in flight together: the
   //    streaming source (periodic wrap included), or for a link entering through a
-  //    side the outgoing population o = opp(q) of this node
+  //    side the outgoing population of this node
   //    (a symmetry side gives the mirrored population of the tangential neighbour)
-  int side[9];
-  bool sym[9];
-  R raw[9];
+  const NodeSides b = node_sides(P, i, j, P.xper, P.yper);
 #pragma unroll
   for (int q = 0; q < 9; q++) {
-    side[q] = entry_side(i, j, cx9(q), cy9(q), P.nx, P.ny, P.xper, P.yper, SYM ? P.fysym : 0);
-    sym[q] = false;
+    const int cx = cx9(q), cy = cy9(q);
+    const bool by_x = enters<SYM>(b, side_x(cx), cx, cy, P.fysym), by_y = enters<SYM>(b, side_y(cy), cx, cy, P.fysym);
+    long long at = by_x || by_y ? opp9(q) * P.plane + n : q * P.plane + stream_at(b, i, cx, cy);
     if (SYM) {
-#pragma unroll
-      for (int s = 0; s < 4; s++)
-        if (side[q] == s) sym[q] = P.side[s].kind == BC_SYMMETRY;
+      if (by_x && P.side[side_x(cx)].kind == BC_SYMMETRY) at = symmetry_source<9>(P, side_x(cx), q, i, j, P.yper);
+      if (by_y && P.side[side_y(cy)].kind == BC_SYMMETRY) at = symmetry_source<9>(P, side_y(cy), q, i, j, P.xper);
     }
-    long long at = side[q] < 0 ? q * P.plane + (long long)wrap(j - cy9(q), P.ny) * P.pitch + wrap(i - cx9(q), P.nx)
-                               : opp9(q) * P.plane + n;
-    if (sym[q]) at = symmetry_source<9>(P, side[q], q, i, j, side[q] >= 2 ? P.xper : P.yper);
-    raw[q] = (R)src[at];
+    f[q] = (R)src[at];
   }
-  // 2. wall / inlet velocities of the sides this node lies on, loaded up front
-  R uws[4][2];
+  // 2. the sides this node lies on: walls and velocity inlets (Eq. BB_vel, f_q = f_o* +
+  //    2 w rho_w c_q.u_w / c_s^2) and the outlet (Eq. anti_BB_vel in deviation form, f_q =
+  //    -f_o* + 2 w [rho_w (1 + (c.u)^2 / 2 c_s^4 - u^2 / 2 c_s^2) - rho0], whose u_w
+  //    extrapolates the pre-collision velocities of time t at the boundary node and its
+  //    inner neighbour)
+  const R ics2 = K<R>(P).inv_cs2;
 #pragma unroll
   for (int s = 0; s < 4; s++) {
-    const double *uw = P.side[s].uw;
-    const bool ld = on_side(P, s, i, j) && uw != nullptr;
-    const int a = along(s, i, j), len = side_len(P, s);
-    uws[s][0] = ld ? (R)uw[a] : (R)0;
-    uws[s][1] = ld ? (R)uw[len + a] : (R)0;
-  }
-  // 3. outlet velocity extrapolation, Eq. anti_BB_vel and the rule below it (reading:
-  //    pre-collision velocities of time t at the boundary node and its inner neighbour)
-  R uwp[4][2];
-#pragma unroll
-  for (int s = 0; s < 4; s++) { uwp[s][0] = 0; uwp[s][1] = 0; }
-#pragma unroll
-  for (int s = 0; s < 4; s++) {
-    if (on_side(P, s, i, j) && P.side[s].kind == BC_PRESSURE) {
-      int ii = i + (s == 0) - (s == 1), jj = j + (s == 2) - (s == 3);
+    if (!b.in[s]) continue;
+    const int kind = P.side[s].kind;
+    if (SYM && kind == BC_SYMMETRY) continue;
+    const R rw = K<R>(P).rho_w[s];
+    R ux = 0, uy = 0, base = 0, lin = 0, quad = 0;
+    const bool anti = kind == BC_PRESSURE;
+    if (anti) {
       R ub, vb, ui, vi;
       post_velocity<S, R>(P, src, i, j, ub, vb);
-      post_velocity<S, R>(P, src, ii, jj, ui, vi);
-      uwp[s][0] = ub + (R)0.5 * (ub - ui);
-      uwp[s][1] = vb + (R)0.5 * (vb - vi);
-    }
-  }
-  // 4. boundary links (side values picked with compile-time side indices)
-#pragma unroll
-  for (int q = 0; q < 9; q++) {
-    if (side[q] < 0 || sym[q]) {
-      f[q] = raw[q];
-      continue;
-    }
-    const int o = opp9(q);
-    const R fo = raw[q];
-    int kind = BC_WALL;
-    R rw = 0, ux = 0, uy = 0;
-#pragma unroll
-    for (int s = 0; s < 4; s++) {
-      if (side[q] == s) {
-        kind = P.side[s].kind;
-        rw = K<R>(P).rho_w[s];
-        ux = kind == BC_PRESSURE ? uwp[s][0] : uws[s][0];
-        uy = kind == BC_PRESSURE ? uwp[s][1] : uws[s][1];
-      }
-    }
-    const R cox = c * (R)cx9(o), coy = c * (R)cy9(o);
-    if (kind == BC_PRESSURE) {
-      // Eq. anti_BB_vel in deviation form: f_q - w rho0 = -(f_o* - w rho0) + 2 w [rho_w(...) - rho0]
-      R cu = cox * ux + coy * uy;
-      R uu = ux * ux + uy * uy;
-      f[q] = -fo + (R)2 * w9<R>(o) * (rw * ((R)1 + (R)0.5 * cu * cu * inv_cs2 * inv_cs2 - (R)0.5 * uu * inv_cs2) - K<R>(P).rho0);
+      post_velocity<S, R>(P, src, i + (s == 0) - (s == 1), j + (s == 2) - (s == 3), ui, vi);
+      ux = ub + (R)0.5 * (ub - ui);
+      uy = vb + (R)0.5 * (vb - vi);
+      base = (R)2 * (rw - K<R>(P).rho0) - rw * (ux * ux + uy * uy) * ics2;
+      quad = rw * ics2 * ics2;
     } else {
-      // Eq. BB_vel (walls and velocity inlet): f_q = f_o* - 2 w_o rho_w c_o.u_w / c_s^2
-      f[q] = fo - (R)2 * w9<R>(o) * rw * (cox * ux + coy * uy) * inv_cs2;
+      const double *uw = P.side[s].uw;
+      if (uw) {
+        const int a = along(s, i, j);
+        ux = (R)uw[a];
+        uy = (R)uw[side_len(P, s) + a];
+      }
+      lin = (R)2 * rw * ics2;
+    }
+#pragma unroll
+    for (int q = 1; q < 9; q++) {
+      if (!enters<SYM>(b, s, cx9(q), cy9(q), P.fysym)) continue;
+      const R cu = K<R>(P).c * ((R)cx9(q) * ux + (R)cy9(q) * uy);
+      f[q] = (anti ? -f[q] : f[q]) + w9<R>(q) * (base + cu * (lin + quad * cu));
     }
   }
 }
@@ -208,85 +232,74 @@ __device__ __forceinline__ void pull_g(const SpParams &P, const S *src, int i, i
     for (int q = 0; q < QT; q++) g[q] = (R)gsrc[q * P.plane + n];
     return;
   }
-  const R c = K<R>(P).c, inv_cs2 = K<R>(P).inv_cs2;
   // 1. gather (branch-free, all loads in flight together)
-  int side[QT], tk[QT];
-  R raw[QT];
+  const NodeSides b = node_sides(P, i, j, P.txper, P.typer);
 #pragma unroll
   for (int q = 0; q < QT; q++) {
-    side[q] = entry_side(i, j, cxT(QT, q), cyT(QT, q), P.nx, P.ny, P.txper, P.typer, SYM ? P.tysym : 0);
-    tk[q] = TBC_NONE;
-#pragma unroll
-    for (int s = 0; s < 4; s++)
-      if (side[q] == s) tk[q] = P.side[s].tkind;
-    long long at;
-    if (side[q] < 0) {
-      at = q * P.plane + (long long)wrap(j - cyT(QT, q), P.ny) * P.pitch + wrap(i - cxT(QT, q), P.nx);
-    } else if (SYM && tk[q] == TBC_SYMMETRY) {
-      at = symmetry_source<QT>(P, side[q], q, i, j, side[q] >= 2 ? P.txper : P.typer);
-    } else if (tk[q] == TBC_OUTFLOW) {
-      // g_q(x_b, t+dt) = g_q(x_b-1, t+dt): the inner node's pull of q (Sec. 2.2, outlet);
+    const int cx = cxT(QT, q), cy = cyT(QT, q);
+    const bool by_x = enters<SYM>(b, side_x(cx), cx, cy, P.tysym), by_y = enters<SYM>(b, side_y(cy), cx, cy, P.tysym);
+    const int tk = by_y ? P.side[side_y(cy)].tkind : P.side[side_x(cx)].tkind;
+    long long at = by_x || by_y ? oppT(QT, q) * P.plane + n : q * P.plane + stream_at(b, i, cx, cy);
+    if ((by_x || by_y) && tk == TBC_OUTFLOW) {
+      // g_q(x_b, t+dt) = g_q(x_b-1, t+dt): the inner node's pull of q (Sec. 2.2, outlet),
+      // whose source is in this node's column (row, for a y-side);
       // where that pull itself crosses a symmetry side (the outlet's corner with a
       // symmetry plane) it is that side's mirrored value
-      const int ii = i + (side[q] == 0) - (side[q] == 1), jj = j + (side[q] == 2) - (side[q] == 3);
-      const int si = ii - cxT(QT, q), sj = jj - cyT(QT, q);
-      at = q * P.plane + (long long)min(max(sj, 0), P.ny - 1) * P.pitch + min(max(si, 0), P.nx - 1);
+      const int si = by_x ? i : min(max(i - cx, 0), P.nx - 1), sj = by_y ? j : min(max(j - cy, 0), P.ny - 1);
+      at = q * P.plane + (long long)sj * P.pitch + si;
       if (SYM) {
-        const int cs = entry_side(ii, jj, cxT(QT, q), cyT(QT, q), P.nx, P.ny, P.txper, P.typer, P.tysym);
+        const int ii = by_x ? i + cx : i, jj = by_y ? j + cy : j;
+        const int cs = entry_side(ii, jj, cx, cy, P.nx, P.ny, P.txper, P.typer, P.tysym);
         bool csym = false;
 #pragma unroll
         for (int s = 0; s < 4; s++)
           if (cs == s) csym = P.side[s].tkind == TBC_SYMMETRY;
         if (csym) at = symmetry_source<QT>(P, cs, q, ii, jj, cs >= 2 ? P.txper : P.typer);
       }
-    } else {
-      at = oppT(QT, q) * P.plane + n;
+    } else if (SYM && (by_x || by_y) && tk == TBC_SYMMETRY) {
+      at = symmetry_source<QT>(P, by_y ? side_y(cy) : side_x(cx), q, i, j, by_y ? P.txper : P.typer);
     }
-    raw[q] = (R)gsrc[at];
+    g[q] = (R)gsrc[at];
   }
-  // 2. wall temperatures / fluxes and velocities of the sides this node lies on
-  R tws[4], uws[4][2];
+  // 2. the sides this node lies on: fixed temperature (Eq. anti_BB_T in deviation form) and
+  //    wall flux (Eq. BB_T, lambda_o = 6 w_o on D2Q9, 1 for the single D2Q5 unknown; zero
+  //    flux = adiabatic).  D2Q5's one weight is folded into the coefficients
+  const R ics2 = K<R>(P).inv_cs2;
+  const R wq = QT == 9 ? (R)1 : w5<R>(1);
+  R wet[2] = {(R)0, (R)0};
 #pragma unroll
   for (int s = 0; s < 4; s++) {
-    const bool on = on_side(P, s, i, j);
-    const double *tw = P.side[s].tw, *uw = P.side[s].uw;
-    const int a = along(s, i, j), len = side_len(P, s);
-    tws[s] = (on && tw) ? (R)tw[a] : (R)0;
-    uws[s][0] = (on && uw) ? (R)uw[a] : (R)0;
-    uws[s][1] = (on && uw) ? (R)uw[len + a] : (R)0;
-  }
-  // 3. boundary links
-#pragma unroll
-  for (int q = 0; q < QT; q++) {
-    if (side[q] < 0 || tk[q] == TBC_OUTFLOW || (SYM && (tk[q] == TBC_SYMMETRY || tk[q] == TBC_WETNODE))) {
-      g[q] = raw[q];
+    if (!b.in[s]) continue;
+    const int a = along(s, i, j), tk = P.side[s].tkind;
+    if (tk == TBC_OUTFLOW || (SYM && tk == TBC_SYMMETRY)) continue;
+    const R tw = P.side[s].tw ? (R)P.side[s].tw[a] : (R)0;
+    if (SYM && tk == TBC_WETNODE) {
+      if (s < 2) wet[s] = tw;
       continue;
     }
-    const int o = oppT(QT, q);
-    const R go = raw[q];
-    R Tw = 0, ux = 0, uy = 0;
-#pragma unroll
-    for (int s = 0; s < 4; s++) {
-      if (side[q] == s) {
-        Tw = tws[s];
-        ux = uws[s][0];
-        uy = uws[s][1];
+    R ux = 0, uy = 0, base, quad = 0;
+    const bool anti = tk == TBC_TEMP;
+    if (anti) {
+      const double *uw = P.side[s].uw;
+      if (uw) {
+        ux = (R)uw[a];
+        uy = (R)uw[side_len(P, s) + a];
       }
-    }
-    if (tk[q] == TBC_TEMP) {
-      // Eq. anti_BB_T in deviation form
-      R cu = c * ((R)cxT(QT, o) * ux + (R)cyT(QT, o) * uy);
-      R uu = ux * ux + uy * uy;
-      g[q] = -go + (R)2 * wT<R>(QT, o) * (Tw * ((R)1 + (R)0.5 * cu * cu * inv_cs2 * inv_cs2 - (R)0.5 * uu * inv_cs2) - K<R>(P).T0);
-    } else if (QT == 9) {
-      // Eq. BB_T with lambda_o = 6 w_o on D2Q9 (4/6 axial, 1/6 diagonal; FLUX, zero flux = adiabatic)
-      g[q] = go + (R)6 * w9<R>(o) * K<R>(P).flux_coef * Tw;
+      base = wq * ((R)2 * (tw - K<R>(P).T0) - tw * (ux * ux + uy * uy) * ics2);
+      quad = wq * (tw * ics2 * ics2);
     } else {
-      // Eq. BB_T with lambda = 1 for the single D2Q5 unknown (FLUX; zero flux = adiabatic)
-      g[q] = go + K<R>(P).flux_coef * Tw;
+      base = (QT == 9 ? (R)6 : (R)1) * K<R>(P).flux_coef * tw;
+    }
+#pragma unroll
+    for (int q = 1; q < QT; q++) {
+      const int cx = cxT(QT, q), cy = cyT(QT, q);
+      if (!enters<SYM>(b, s, cx, cy, P.tysym)) continue;
+      const R cu = K<R>(P).c * ((R)cx * ux + (R)cy * uy);
+      const R v = base + quad * cu * cu;
+      g[q] = (anti ? -g[q] : g[q]) + (QT == 9 ? w9<R>(q) * v : v);
     }
   }
-  // 4. wet-node x-sides (App. B, Eq. BCs_1D_advection_diffusion): the boundary node lies
+  // 3. wet-node x-sides (App. B, Eq. BCs_1D_advection_diffusion): the boundary node lies
   //    on the boundary; its single D2Q5 unknown closes T of Eq. zero_moment_g at T_w,
   //    g_unknown = T_w - dt qdot/2 - (sum of the others), in deviation form
   if (SYM && QT == 5) {
@@ -299,7 +312,7 @@ __device__ __forceinline__ void pull_g(const SpParams &P, const S *src, int i, i
       for (int k = 0; k < QT; k++)
         if (k != qu) others += g[k];
       const R qd = P.qdot ? (R)((const S *)P.qdot)[n] : (R)0;
-      g[qu] = (tws[s] - K<R>(P).T0) - (R)0.5 * K<R>(P).dt * qd - others;
+      g[qu] = (wet[s] - K<R>(P).T0) - (R)0.5 * K<R>(P).dt * qd - others;
     }
   }
 }

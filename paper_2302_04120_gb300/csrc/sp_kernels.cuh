@@ -50,15 +50,15 @@ __device__ __forceinline__ void step_node(const SpParams &P, int i, int j) {
 __device__ __forceinline__ bool frame_node(int nx, int ny, int f, int &i, int &j) {
   const int rows = ny >= 2 ? 2 : 1, cols = nx >= 2 ? 2 : 1;
   if (f < rows * nx) {
-    i = f % nx;
-    j = (f / nx) ? ny - 1 : 0;
+    i = f < nx ? f : f - nx;
+    j = f < nx ? 0 : ny - 1;
     return true;
   }
   f -= rows * nx;
   const int inner = ny - 2;
   if (inner <= 0 || f >= cols * inner) return false;
-  i = (f / inner) ? nx - 1 : 0;
-  j = 1 + f % inner;
+  i = f < inner ? 0 : nx - 1;
+  j = 1 + (f < inner ? f : f - inner);
   return true;
 }
 
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(256) k_init(const SpParams P, const double *A,
 
 // Macroscopic fields of the current time: pull (with boundary rules) + moments.
 template <int PREC, int FLOW, int TH, bool SYM>
-__global__ void __launch_bounds__(256) k_moments(const SpParams P, unsigned mask, double *out) {
+__global__ void __launch_bounds__(256, PREC == 1 ? 3 : 2) k_moments(const SpParams P, unsigned mask, double *out) {
   typedef typename Prec<PREC>::S S;
   typedef typename Prec<PREC>::R R;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;

@@ -160,11 +160,16 @@ __device__ __forceinline__ void step_node_staged(const SpParams &P, int i, int j
   }
 }
 
+// Resident CTAs per SM that the register budget leaves room for (lbm_set_launch accepts
+// as many as fit): 128 registers a thread, 40 without a momentum lattice.
+template <int FLOW, int TY>
+constexpr int min_ctas() { return (FLOW != FLOW_NONE ? 2 : 6) * (8 / TY); }
+
 template <int PREC, int FLOW, int TH, int TY>
 // wait_ns: wall-time limit of each ring wait.  expire_probe (self-test of the timeout
 // path): each block first waits, with that limit, on a barrier of its own that nothing
 // completes, so the wait runs out and the block takes the failure path below.
-__global__ void __launch_bounds__(kTileX *TY) k_step_tma(const SpParams P, const __grid_constant__ CUtensorMap map,
+__global__ void __launch_bounds__(kTileX *TY, min_ctas<FLOW, TY>()) k_step_tma(const SpParams P, const __grid_constant__ CUtensorMap map,
                                                          int ntx, int ntiles, int nstages, int *flag,
                                                          unsigned long long wait_ns, int expire_probe) {
   typedef typename Prec<PREC>::S S;
