@@ -397,7 +397,7 @@ def _roofline_d2q9(steps, warmup, stream, torch, launch=None):
     return {"workload": "poiseuille_d2q9_bgk_8192x4096", "bound": "hbm", "value": round(n / t / 1e6, 1),
             "unit_value": "MLUPS", "achieved": round(72 * n / t / 1e9, 1), "peak": peak, "unit": "GB/s",
             "frac": round(72 * n / t / 1e9 / peak, 4), "steps": steps, "status": int(chk),
-            "kernel": "k_step_split<1,FLOW_BGK,TH_NONE>", "launch": _launch_desc(cfg),
+            "kernel": "k_step_split<1,FLOW_MRT,TH_NONE>", "launch": _launch_desc(cfg),
             "l2": "state 2.4 GB, larger than L2; back-to-back steps"}
 
 

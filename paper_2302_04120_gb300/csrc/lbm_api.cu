@@ -153,6 +153,21 @@ static void fill_const(const SpParams &P, lbmk::SpConst<R> &k) {
   k.omega = (R)P.omega; k.s_e = (R)P.s_e; k.s_eps = (R)P.s_eps; k.s_q = (R)P.s_q; k.s_nu = (R)P.s_nu;
   k.omegaT = (R)P.omegaT; k.tsrc_fac = (R)P.tsrc_fac; k.flux_coef = (R)P.flux_coef;
   k.bgx = (R)P.bgx; k.bgy = (R)P.bgy; k.T_ref = (R)P.T_ref;
+  const double f_e = (1.0 - 0.5 * P.s_e) * P.dt, f_eps = (1.0 - 0.5 * P.s_eps) * P.dt;
+  const double f_q = (1.0 - 0.5 * P.s_q) * P.dt, f_nu = (1.0 - 0.5 * P.s_nu) * P.dt;
+  k.hdt_ic = (R)(0.5 * P.dt / P.c);
+  k.kq = (R)(P.s_q / 6.0);
+  k.kn = (R)(0.25 * P.s_nu);
+  k.ke = (R)(P.s_e / 36.0);
+  k.kep = (R)(P.s_eps / 12.0);
+  k.gq = (R)((f_q + P.dt) / 6.0);
+  k.gd = (R)(P.dt / 6.0 - f_q / 12.0);
+  k.gn = (R)(0.5 * f_nu);
+  k.g4 = (R)((2.0 * f_eps - f_e) / 6.0);
+  k.g8 = (R)((2.0 * f_e - f_eps) / 6.0);
+  k.hsT = (R)(0.5 * P.omegaT);
+  k.q1T = (R)((1.0 + P.omegaT) / 6.0);
+  k.q2T = (R)(0.25 * P.omegaT);
   for (int s = 0; s < 4; s++) k.rho_w[s] = (R)P.side[s].rho_w;
 }
 
@@ -187,6 +202,8 @@ static SpParams sp_params(const lbm_t h, int from_buf) {
   const double wnu = 1.0 / h->tau;
   const double wq = (3.0 / p.dt) * (2.0 / p.dt - wnu) / (3.0 / p.dt - wnu);
   P.s_e = p.omega_e_dt; P.s_eps = p.omega_eps_dt; P.s_q = wq * p.dt; P.s_nu = wnu * p.dt;
+  if (p.flow_op == LBM_BGK) P.s_e = P.s_eps = P.s_q = P.s_nu = P.omega;  // BGK: one rate
+  P.unit_e = P.s_e == 1.0 && P.s_eps == 1.0;
   if (p.thermal) {
     P.omegaT = p.dt / h->tauT;
     const double tau_sg = (p.literal & 1) ? h->tau : h->tauT;  // reading R1
@@ -201,6 +218,7 @@ static SpParams sp_params(const lbm_t h, int from_buf) {
   }
   P.qdot = h->sink_conv != 0.0 ? h->d_qs[1 - from_buf] : h->d_qdot;
   P.force = h->d_force;
+  P.forced = P.Fx != 0.0 || P.Fy != 0.0 || P.force || P.buoy;
   fill_const(P, P.kd);
   fill_const(P, P.kf);
   P.local = h->pre;
@@ -361,7 +379,7 @@ extern "C" lbm_status lbm_create(const lbm_params *pin, void *stream, lbm_t *out
   h->tmap_ty = 0;
   h->last_good = -1;
   if (!p.phase && (p.flow || p.thermal)) {
-    int fk = p.flow ? (p.flow_op == LBM_MRT ? lbmk::FLOW_MRT : lbmk::FLOW_BGK) : lbmk::FLOW_NONE;
+    int fk = p.flow ? lbmk::FLOW_MRT : lbmk::FLOW_NONE;
     int tk = th_kind(p);
     lbmk::sp_tma_prepare(p.precision, fk, tk);  // failure leaves only the grid launch usable
     cudaGetLastError();
@@ -580,7 +598,7 @@ extern "C" lbm_status lbm_init_fields(lbm_t h, const double *a, const double *ux
     e = lbmk::mp_init(P, h->p.precision, d_in[0], d_in[1], d_in[2], d_in[3], h->stream);
   } else {
     SpParams P = sp_params(h, 1);
-    int flow = h->p.flow ? (h->p.flow_op == LBM_MRT ? lbmk::FLOW_MRT : lbmk::FLOW_BGK) : lbmk::FLOW_NONE;
+    int flow = h->p.flow ? lbmk::FLOW_MRT : lbmk::FLOW_NONE;
     int th = th_kind(h->p);
     e = lbmk::sp_init(P, h->p.precision, flow, th, d_in[0], d_in[1], d_in[2], d_in[3], h->block, h->stream);
   }
@@ -599,7 +617,7 @@ extern "C" lbm_status lbm_init_fields(lbm_t h, const double *a, const double *ux
 }
 
 static void sp_kinds(const lbm_t h, int *flow, int *th) {
-  *flow = h->p.flow ? (h->p.flow_op == LBM_MRT ? lbmk::FLOW_MRT : lbmk::FLOW_BGK) : lbmk::FLOW_NONE;
+  *flow = h->p.flow ? lbmk::FLOW_MRT : lbmk::FLOW_NONE;
   *th = th_kind(h->p);
 }
 

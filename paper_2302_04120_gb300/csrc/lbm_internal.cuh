@@ -26,6 +26,11 @@ struct SpConst {
   R hdt;                            // dt / 2
   R fk_e, fk_eps, fk_q, fk_nu;      // MRT forcing factors (1 - s_k / 2) dt, s_k = dt Lambda_k
   R omega, s_e, s_eps, s_q, s_nu, omegaT, tsrc_fac, flux_coef, bgx, bgy, T_ref;
+  // folded factors of the pair-form collisions (sp_device.cuh), formed in FP64:
+  R hdt_ic;                         // dt / (2 c)
+  R kq, kn, ke, kep;                // s_q / 6, s_nu / 4, s_e / 36, s_eps / 12
+  R gq, gd, gn, g4, g8;             // forcing: axis and diagonal odd pairs, stress, energies
+  R hsT, q1T, q2T;                  // omegaT / 2, (1 + omegaT) / 6, omegaT / 4
   R rho_w[4];
 };
 
@@ -48,8 +53,10 @@ struct SpParams {
   double Fx, Fy;          // uniform body force
   double ux_pres, uy_pres;
   // momentum collision
-  double omega;           // BGK: dt/tau
-  double s_e, s_eps, s_q, s_nu;  // MRT: dt * Lambda_k for e, eps, q, nu moments
+  double omega;           // dt/tau
+  double s_e, s_eps, s_q, s_nu;  // dt * Lambda_k for e, eps, q, nu moments (BGK: all dt/tau)
+  int unit_e;             // s_e = s_eps = 1: these two moments go to equilibrium
+  int forced;             // a body force, a force field or buoyancy acts
   // thermal collision
   double omegaT;          // dt/tau_T
   double tsrc_fac;        // BGK thermal source prefactor (1 - dt/(2 tau_sg))
@@ -75,7 +82,7 @@ __device__ __forceinline__ const SpConst<double> &K<double>(const SpParams &P) {
 template <>
 __device__ __forceinline__ const SpConst<float> &K<float>(const SpParams &P) { return P.kf; }
 
-enum { FLOW_NONE = 0, FLOW_BGK = 1, FLOW_MRT = 2 };
+enum { FLOW_NONE = 0, FLOW_MRT = 2 };  // momentum BGK: the MRT kernels with equal rates
 
 // Nodes of the boundary frame of an nx x ny grid: rows j = 0 and ny - 1, then the
 // columns i = 0 and nx - 1 between them (each node once, also for nx or ny < 3).

@@ -320,11 +320,41 @@ __device__ __forceinline__ void pull_g(const SpParams &P, const S *src, int i, i
 // ----------------------------------------------------------------------------
 // Moments and collisions (deviation form)
 // ----------------------------------------------------------------------------
+// The collisions work on pairs of opposite populations: with a = f_q + f_opp and
+// d = f_q - f_opp, a pair changes by (dP + dQ, dP - dQ), dP the change of its even
+// moments and dQ of its odd ones.  On the pairs every MRT operator of Sec. 2.1 / 2.2 is a
+// handful of products (the same operator as M^-1 Lambda M, with factors folded on the host
+// into SpConst).  The changes are formed from the small non-equilibrium parts and added to
+// the populations once, so that a population is rounded once per step, and the conserved
+// moments are kept by construction.
+// Why in this form: on GB300 the FP64 pipe issues one warp instruction every 16 cycles
+// per SM and bounds the FP64 step, so the count of FP64 instructions per node is its
+// time.  The unfolded form (moments, equilibria and forcing of all nine rates, then
+// M^-1) took 198 per node of D2Q9 MRT + D2Q5 MRT, this one about 90.  Measured, back-to-back
+// steps: FP64 2048 x 256 191.6 -> 102.4 us, FP64 64 x 33 BGK 14.6 -> 8.5 us, FP32 2048 x 256
+// 10.1 -> 9.1 us; the error against a 64-bit solution is not larger in either precision.
 template <typename R>
 struct Macro {
   R drho, rho, ux, uy, Fx, Fy;  // momentum
-  R sumg, qd, T;                // thermal
+  R hx, hy, jx, jy;             // lattice-scaled: u / c and rho u / c
+  R sumg, qd, dT, T;            // thermal; dT = T - T0
 };
+
+// 1 / x for a normal x: the hardware's approximate reciprocal and the third-order
+// iteration r (1 + e + e^2), e = 1 - x r (second order in FP32, whose seed already has
+// 23 bits).  Two to four instructions instead of the IEEE division's sequence; within
+// one unit in the last place.
+__device__ __forceinline__ float recip(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return fmaf(r, fmaf(-x, r, 1.0f), r);
+}
+__device__ __forceinline__ double recip(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
 
 template <typename S, typename R>
 __device__ __forceinline__ void load_sources(const SpParams &P, long long n, Macro<R> &m) {
@@ -338,254 +368,217 @@ __device__ __forceinline__ void load_sources(const SpParams &P, long long n, Mac
   m.qd = P.qdot ? (R)((const S *)P.qdot)[n] : (R)0;
 }
 
+// Sums over a lattice's populations that moments and collisions share (written once, so
+// that both use the same instructions): s14 = f1 + .. + f4, s58 = f5 + .. + f8 and the
+// lattice-scaled first moment.
+template <typename R>
+__device__ __forceinline__ R sum14(const R *f) { return (f[1] + f[3]) + (f[2] + f[4]); }
+template <typename R>
+__device__ __forceinline__ R sum58(const R *f) { return (f[5] + f[7]) + (f[6] + f[8]); }
+template <typename R>
+__device__ __forceinline__ R first_x9(const R *f) { return (f[1] - f[3]) + ((f[5] - f[7]) - (f[6] - f[8])); }
+template <typename R>
+__device__ __forceinline__ R first_y9(const R *f) { return (f[2] - f[4]) + ((f[5] - f[7]) + (f[6] - f[8])); }
+
 template <typename R, int FLOW, int TH>
 __device__ __forceinline__ void moments(const SpParams &P, const R f[9], const R *g, Macro<R> &m) {
   if (TH != TH_NONE) {
     // Eq. zero_moment_g
-    if (ThLat<TH>::Q == 9) m.sumg = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
-    else m.sumg = (g[0] + g[1]) + (g[2] + g[3]) + g[4];
-    m.T = K<R>(P).T0 + m.sumg + K<R>(P).hdt * m.qd;
+    m.sumg = ThLat<TH>::Q == 9 ? g[0] + (sum14(g) + sum58(g)) : g[0] + sum14(g);
+    m.dT = m.sumg;
+    if (P.qdot) m.dT += K<R>(P).hdt * m.qd;
+    m.T = K<R>(P).T0 + m.dT;
     if (FLOW != FLOW_NONE && P.buoy) {
       // Boussinesq buoyancy with this step's temperature (Eq. buoyancy_force)
-      const R dT = (K<R>(P).T0 - K<R>(P).T_ref) + m.sumg + K<R>(P).hdt * m.qd;
+      const R dT = (K<R>(P).T0 - K<R>(P).T_ref) + m.dT;
       m.Fx += K<R>(P).bgx * dT;
       m.Fy += K<R>(P).bgy * dT;
     }
   }
   if (FLOW != FLOW_NONE) {
     // Eqs. zero_moment_f and first_moment_f
-    m.drho = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
+    m.drho = f[0] + (sum14(f) + sum58(f));
     m.rho = K<R>(P).rho0 + m.drho;
-    const R c = K<R>(P).c, hdt = K<R>(P).hdt;
-    const R jx = c * ((f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]));
-    const R jy = c * ((f[2] - f[4]) + (f[5] - f[8]) + (f[6] - f[7]));
-    const R inv = (R)1 / m.rho;
-    m.ux = (jx + hdt * m.Fx) * inv;
-    m.uy = (jy + hdt * m.Fy) * inv;
+    m.jx = first_x9(f);
+    m.jy = first_y9(f);
+    if (P.forced) {
+      m.jx += K<R>(P).hdt_ic * m.Fx;
+      m.jy += K<R>(P).hdt_ic * m.Fy;
+    }
+    const R inv = recip(m.rho);
+    m.hx = m.jx * inv;
+    m.hy = m.jy * inv;
+    m.ux = K<R>(P).c * m.hx;
+    m.uy = K<R>(P).c * m.hy;
   } else {
     m.drho = 0;
     m.rho = K<R>(P).rho0;
     m.ux = K<R>(P).ux_pres;
     m.uy = K<R>(P).uy_pres;
+    m.hx = m.ux * K<R>(P).inv_c;
+    m.hy = m.uy * K<R>(P).inv_c;
   }
 }
 
+// Momentum collision: MRT (Eq. colisao_MRT, [M]_dim of Eq. M_matrix_dim, Guo forcing),
+// and BGK as the MRT whose rates all equal dt / tau (set on the host).  With
+// h = u / c, j = rho h:
+//   even moments   stress: s_nu times the distance of the pair differences from
+//                  rho h_x^2 - rho h_y^2 and rho h_x h_y; energy and energy square: at
+//                  rate 1 (unit_e) to the equilibrium, else relaxed by the distances of
+//                  the two moments (over 1 and 3) from their equilibria;
+//   odd moments    axis pairs: (s_q / 6)(t + j - 2 d), t the diagonals' share of the first
+//                  moment; diagonal pairs: minus half of that, which keeps the momentum.
 template <typename R>
-__device__ __forceinline__ void collide_bgk9(const SpParams &P, const Macro<R> &m, R f[9]) {
-  const R c = K<R>(P).c, inv_cs2 = K<R>(P).three_inv_c2, inv_cs4 = inv_cs2 * inv_cs2;
-  const R om = K<R>(P).omega;
-  const R fac = ((R)1 - (R)0.5 * om) * K<R>(P).dt;  // (1 - dt/(2 tau)) dt
-  const R hu = (R)0.5 * (m.ux * m.ux + m.uy * m.uy) * inv_cs2;  // u^2 / (2 c_s^2)
-  const R uF = m.ux * m.Fx + m.uy * m.Fy;
-  // q >= 1 first; the rest population takes the remainders so that sum f_eq = rho
-  // and sum F_hat = 0 hold exactly in the working precision (the rounded weights
-  // do not sum to one in FP32)
-  R feq_sum = 0, fh_sum = 0;
-#pragma unroll
-  for (int q = 1; q < 9; q++) {
-    const R cxq = c * (R)cx9(q), cyq = c * (R)cy9(q);
-    const R cu = cxq * m.ux + cyq * m.uy;
-    // f_eq - w rho0 (Eq. feq_geral, deviation form: no O(rho0) cancellation)
-    const R feq = w9<R>(q) * (m.drho + m.rho * (cu * inv_cs2 * ((R)1 + (R)0.5 * cu * inv_cs2) - hu));
-    // Guo forcing F_hat (Eq. forcing_term)
-    const R cF = cxq * m.Fx + cyq * m.Fy;
-    const R Fh = w9<R>(q) * ((cF - uF) * inv_cs2 + cu * cF * inv_cs4);
-    feq_sum += feq;
-    fh_sum += Fh;
-    f[q] = f[q] - om * (f[q] - feq) + fac * Fh;
+__device__ __forceinline__ void collide_flow(const SpParams &P, const Macro<R> &m, R f[9]) {
+  const SpConst<R> &k = K<R>(P);
+  const R d13 = f[1] - f[3], d24 = f[2] - f[4], d57 = f[5] - f[7], d68 = f[6] - f[8];
+  const R a13 = f[1] + f[3], a24 = f[2] + f[4], a57 = f[5] + f[7], a68 = f[6] + f[8];
+  const R s14 = a13 + a24, s58 = a57 + a68;
+  const R xx0 = m.jx * m.hx, ru = xx0 + m.jy * m.hy, rxx = xx0 - m.jy * m.hy, rxy = m.jx * m.hy;
+  R dX = k.kn * (rxx - (a13 - a24)), dY = k.kn * (rxy - (a57 - a68));
+  R ox = k.kq * (((d57 - d68) + m.jx) - (R)2 * d13);
+  R oy = k.kq * (((d57 + d68) + m.jy) - (R)2 * d24);
+  R d4, d8;  // change of every axis and of every diagonal population's share of the energies
+  R f0;
+  if (P.unit_e) {
+    const R r12 = ru * ((R)1 / (R)12);
+    const R e4 = m.drho * ((R)1 / (R)9) + r12, e8 = m.drho * ((R)1 / (R)36) + r12;
+    d4 = e4 - (R)0.25 * s14;
+    d8 = e8 - (R)0.25 * s58;
+    f0 = m.drho - (R)4 * (e4 + e8);
+  } else {
+    const R a1 = k.ke * (((s14 - (R)2 * f[0]) + (R)4 * s58) - (R)3 * ru), a2 = k.kep * ((f[0] - s14) + ru);
+    d4 = a1 + (R)2 * a2;
+    d8 = -((R)2 * a1 + a2);
+    f0 = f[0] + (R)4 * (a1 - a2);
   }
-  f[0] = f[0] - om * (f[0] - (m.drho - feq_sum)) + fac * (-fh_sum);
+  R w = (R)0.5 * (oy + ox), v = (R)0.5 * (oy - ox);
+  if (P.forced) {
+    const R px = m.Fx * k.inv_c, py = m.Fy * k.inv_c, uF = m.hx * px + m.hy * py;
+    dX += k.gn * (m.hx * px - m.hy * py);
+    dY += (R)0.5 * k.gn * (m.hx * py + m.hy * px);
+    ox += k.gq * px;
+    oy += k.gq * py;
+    w -= k.gd * (py + px);
+    v -= k.gd * (py - px);
+    d4 += k.g4 * uF;
+    d8 += k.g8 * uF;
+    f0 -= (R)4 * ((k.g4 + k.g8) * uF);
+  }
+  const R p13 = d4 + dX, p24 = d4 - dX, p57 = d8 + dY, p68 = d8 - dY;
+  f[0] = f0;
+  f[1] += p13 + ox;
+  f[3] += p13 - ox;
+  f[2] += p24 + oy;
+  f[4] += p24 - oy;
+  f[5] += p57 - w;
+  f[7] += p57 + w;
+  f[6] += p68 - v;
+  f[8] += p68 + v;
 }
 
+// d - T h without rounding the absolute temperature (T0 and T - T0 apart).
 template <typename R>
-__device__ __forceinline__ void collide_mrt9(const SpParams &P, const Macro<R> &m, R f[9]) {
-  const R c = K<R>(P).c, ic = K<R>(P).inv_c;
-  const R dt = K<R>(P).dt;
-  // lattice-scaled moments of the deviations (rows of Eq. M_matrix)
-  const R s14 = (f[1] + f[2]) + (f[3] + f[4]);
-  const R s58 = (f[5] + f[6]) + (f[7] + f[8]);
-  const R m_e = -(R)4 * f[0] - s14 + (R)2 * s58;
-  const R m_ep = (R)4 * f[0] - (R)2 * s14 + s58;
-  const R d58 = (f[5] - f[7]), d68 = (f[6] - f[8]);
-  const R m_qx = (R)2 * (f[3] - f[1]) + d58 - d68;
-  const R m_qy = (R)2 * (f[4] - f[2]) + d58 + d68;
-  const R m_xx = (f[1] + f[3]) - (f[2] + f[4]);
-  const R m_xy = (f[5] + f[7]) - (f[6] + f[8]);
-  // equilibrium and forcing moments divided by c^n (Eq. M_matrix_dim row orders)
-  const R ux = m.ux * ic, uy = m.uy * ic, usq = ux * ux + uy * uy;
-  const R Fx = m.Fx * ic, Fy = m.Fy * ic, uF = ux * Fx + uy * Fy;
-  const R eq_e = -(R)2 * m.drho + (R)3 * m.rho * usq;
-  const R eq_ep = m.drho - (R)3 * m.rho * usq;
-  const R eq_qx = -m.rho * ux, eq_qy = -m.rho * uy;
-  const R eq_xx = m.rho * (ux * ux - uy * uy), eq_xy = m.rho * ux * uy;
-  const R s_e = K<R>(P).s_e, s_ep = K<R>(P).s_eps, s_q = K<R>(P).s_q, s_nu = K<R>(P).s_nu;
-  // Delta m_k = dt Lambda_k (m_k - m_k^eq) - dt (1 - dt Lambda_k / 2) F_k  (Eq. colisao_MRT)
-  // (the factors (1 - dt Lambda_k / 2) dt come from the host-filled constants)
-  const R d_e = s_e * (m_e - eq_e) - K<R>(P).fk_e * ((R)6 * uF);
-  const R d_ep = s_ep * (m_ep - eq_ep) + K<R>(P).fk_eps * ((R)6 * uF);
-  const R d_jx = -dt * Fx, d_jy = -dt * Fy;
-  const R d_qx = s_q * (m_qx - eq_qx) + K<R>(P).fk_q * Fx;
-  const R d_qy = s_q * (m_qy - eq_qy) + K<R>(P).fk_q * Fy;
-  const R d_xx = s_nu * (m_xx - eq_xx) - K<R>(P).fk_nu * ((R)2 * (ux * Fx - uy * Fy));
-  const R d_xy = s_nu * (m_xy - eq_xy) - K<R>(P).fk_nu * (ux * Fy + uy * Fx);
-  // back to populations: M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4)
-  const R a1 = d_e * ((R)1 / (R)36), a2 = d_ep * ((R)1 / (R)36);
-  const R a3 = d_jx * ((R)1 / (R)6), a4 = d_qx * ((R)1 / (R)12);
-  const R a5 = d_jy * ((R)1 / (R)6), a6 = d_qy * ((R)1 / (R)12);
-  const R a7 = d_xx * (R)0.25, a8 = d_xy * (R)0.25;
-  const R ax = -a1 - (R)2 * a2;   // common to i = 1..4
-  const R dg = (R)2 * a1 + a2;    // common to i = 5..8
-  f[0] -= (R)4 * (a2 - a1);
-  f[1] -= ax + a3 - (R)2 * a4 + a7;
-  f[2] -= ax + a5 - (R)2 * a6 - a7;
-  f[3] -= ax - a3 + (R)2 * a4 + a7;
-  f[4] -= ax - a5 + (R)2 * a6 - a7;
-  const R p34 = a3 + a4, p56 = a5 + a6;
-  f[5] -= dg + p34 + p56 + a8;
-  f[6] -= dg - p34 + p56 - a8;
-  f[7] -= dg - p34 - p56 + a8;
-  f[8] -= dg + p34 - p56 - a8;
+__device__ __forceinline__ R off_eq(const Macro<R> &m, R T0, R d, R h) { return (d - T0 * h) - m.dT * h; }
+
+// Thermal BGK with source (Eqs. eq_lattice_boltzmann_BGK_T, forcing_term_g, geq_geral)
+// on the thermal lattice QT: even pairs by w (omega dT + src) - (omega / 2) a, odd pairs
+// by -(omega / 2)(d - d_eq), rest population from the remainder.
+template <typename R, int QT>
+__device__ __forceinline__ void collide_bgk_T(const SpParams &P, const Macro<R> &m, R *g) {
+  const SpConst<R> &k = K<R>(P);
+  const R d13 = g[1] - g[3], d24 = g[2] - g[4], a13 = g[1] + g[3], a24 = g[2] + g[4];
+  const R om = k.omegaT, ho = k.hsT;
+  R b = om * m.dT, dS = (R)0;
+  if (P.qdot) {
+    const R src = k.tsrc_fac * k.dt * m.qd;
+    b += src;
+    dS = om * (k.hdt * m.qd) + src;  // sum g changes by the source alone
+  }
+  if (QT == 5) {
+    const R b6 = b * ((R)1 / (R)6);
+    const R px = b6 - ho * a13, py = b6 - ho * a24;
+    const R ox = ho * off_eq(m, k.T0, d13, m.hx), oy = ho * off_eq(m, k.T0, d24, m.hy);
+    g[0] += dS - (R)2 * (px + py);
+    g[1] += px - ox;
+    g[3] += px + ox;
+    g[2] += py - oy;
+    g[4] += py + oy;
+    return;
+  }
+  // D2Q9: equilibrium differences (2/3) T h on the axes, T (h_y +- h_x) / 6 on the diagonals
+  const R d57 = g[5] - g[7], d68 = g[6] - g[8], a57 = g[5] + g[7], a68 = g[6] + g[8];
+  const R b9 = b * ((R)1 / (R)9), b36 = b * ((R)1 / (R)36);
+  const R p13 = b9 - ho * a13, p24 = b9 - ho * a24, p57 = b36 - ho * a57, p68 = b36 - ho * a68;
+  const R hx = m.hx * ((R)2 / (R)3), hy = m.hy * ((R)2 / (R)3);
+  const R ha = (m.hy + m.hx) * ((R)1 / (R)6), hb = (m.hy - m.hx) * ((R)1 / (R)6);
+  const R o13 = ho * off_eq(m, k.T0, d13, hx), o24 = ho * off_eq(m, k.T0, d24, hy);
+  const R o57 = ho * off_eq(m, k.T0, d57, ha), o68 = ho * off_eq(m, k.T0, d68, hb);
+  g[0] += dS - (R)2 * ((p13 + p24) + (p57 + p68));
+  g[1] += p13 - o13;
+  g[3] += p13 + o13;
+  g[2] += p24 - o24;
+  g[4] += p24 + o24;
+  g[5] += p57 - o57;
+  g[7] += p57 + o57;
+  g[6] += p68 - o68;
+  g[8] += p68 + o68;
 }
 
-// Thermal BGK with source (Eqs. eq_lattice_boltzmann_BGK_T, forcing_term_g,
-// geq_geral) on the thermal lattice QT.
-template <typename R, int QT = 5>
-__device__ __forceinline__ void collide_bgk5(const SpParams &P, const Macro<R> &m, R *g) {
-  const R c = K<R>(P).c, inv_cs2 = K<R>(P).three_inv_c2;
-  const R om = K<R>(P).omegaT;
-  const R src = K<R>(P).tsrc_fac * K<R>(P).dt * m.qd;
-  const R dT = m.T - K<R>(P).T0;
-  R geq_sum = 0, s_sum = 0;
-#pragma unroll
-  for (int q = 1; q < QT; q++) {
-    const R cu = c * ((R)cxT(QT, q) * m.ux + (R)cyT(QT, q) * m.uy);
-    const R geq = wT<R>(QT, q) * (dT + m.T * cu * inv_cs2);  // Eq. geq_geral minus w T0
-    const R sq = wT<R>(QT, q) * src;                         // Eq. forcing_term_g
-    geq_sum += geq;
-    s_sum += sq;
-    g[q] = g[q] - om * (g[q] - geq) + sq;
-  }
-  // rest population from the remainders: sum g_eq = T - T0, sum S = source, exactly
-  g[0] = g[0] - om * (g[0] - (dT - geq_sum)) + (src - s_sum);
+// Thermal MRT on D2Q5: moments (1, c_x, c_y, 5|c|^2 - 4c^2, c_x^2 - c_y^2), rates
+// (0, 1/tau_T, 1/tau_T, 1/dt, 1/dt), source Delta t (I - dt Lambda/2) M (w qdot).  The two
+// even moments at rate 1/dt leave every even pair at w S, S = sum g + dt qdot.
+template <typename R>
+__device__ __forceinline__ void collide_mrt5(const SpParams &P, const Macro<R> &m, R g[5]) {
+  const SpConst<R> &k = K<R>(P);
+  const R d13 = g[1] - g[3], d24 = g[2] - g[4], a13 = g[1] + g[3], a24 = g[2] + g[4];
+  const R S = P.qdot ? m.sumg + k.dt * m.qd : m.sumg;
+  const R p = S * ((R)1 / (R)6);
+  const R px = p - (R)0.5 * a13, py = p - (R)0.5 * a24;
+  const R ex = off_eq(m, k.T0, d13, m.hx), ey = off_eq(m, k.T0, d24, m.hy);
+  g[0] = S - (R)4 * p;
+  g[1] += px - k.hsT * ex;
+  g[3] += px + k.hsT * ex;
+  g[2] += py - k.hsT * ey;
+  g[4] += py + k.hsT * ey;
 }
 
 // Thermal MRT on D2Q9 (Sec. 2.2): the momentum transformation matrices and
 // [Lambda_T] = diag(0, 1, 1, omega_T, 1, omega_T, 1, 1, 1), the unit rates read as
-// 1/dt; source Delta t (I - dt Lambda/2) M (w qdot).  Lattice-scaled moments of the
-// deviations g - w T0; equilibrium moments of g_eq - w T0 from Eq. geq_geral:
-// (T - T0, -2 (T - T0), T - T0, T u_x/c, -T u_x/c, T u_y/c, -T u_y/c, 0, 0).
+// 1/dt; source Delta t (I - dt Lambda/2) M (w qdot).  Every even pair goes to w S,
+// S = sum g + dt qdot; of the odd moments the first loses s_T of its distance e = j - T h
+// from equilibrium, the third-order ones go to -T h.
 template <typename R>
 __device__ __forceinline__ void collide_mrt9T(const SpParams &P, const Macro<R> &m, R g[9]) {
-  const R ic = K<R>(P).inv_c, dt = K<R>(P).dt;
-  const R dT = m.T - K<R>(P).T0;
-  const R sT = K<R>(P).omegaT;  // dt / tau_T
-  const R qd = m.qd;
-  const R s14 = (g[1] + g[2]) + (g[3] + g[4]);
-  const R s58 = (g[5] + g[6]) + (g[7] + g[8]);
-  const R m_e = -(R)4 * g[0] - s14 + (R)2 * s58;
-  const R m_ep = (R)4 * g[0] - (R)2 * s14 + s58;
-  const R d58 = g[5] - g[7], d68 = g[6] - g[8];
-  const R m_jx = (g[1] - g[3]) + d58 - d68;
-  const R m_jy = (g[2] - g[4]) + d58 + d68;
-  const R m_qx = (R)2 * (g[3] - g[1]) + d58 - d68;
-  const R m_qy = (R)2 * (g[4] - g[2]) + d58 + d68;
-  const R m_xx = (g[1] + g[3]) - (g[2] + g[4]);
-  const R m_xy = (g[5] + g[7]) - (g[6] + g[8]);
-  const R Tux = m.T * m.ux * ic, Tuy = m.T * m.uy * ic;
-  // Delta m_k = dt Lambda_k (m_k - m_k^eq) - dt (1 - dt Lambda_k / 2) S_k, S = qdot (1, -2, 1, 0, ...)
-  const R d0 = -dt * qd;                                       // Lambda_0 = 0
-  const R d_e = (m_e + (R)2 * dT) + dt * qd;                   // rate 1/dt: -(dt/2)(-2 qdot)
-  const R d_ep = (m_ep - dT) - (R)0.5 * dt * qd;
-  const R d_jx = sT * (m_jx - Tux), d_jy = sT * (m_jy - Tuy);  // rate omega_T
-  const R d_qx = m_qx + Tux, d_qy = m_qy + Tuy;                // rate 1/dt, eq -T u/c
-  const R d_xx = m_xx, d_xy = m_xy;                            // rate 1/dt, eq 0
-  // back to populations: M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4)
-  const R a0 = d0 * ((R)1 / (R)9);
-  const R a1 = d_e * ((R)1 / (R)36), a2 = d_ep * ((R)1 / (R)36);
-  const R a3 = d_jx * ((R)1 / (R)6), a4 = d_qx * ((R)1 / (R)12);
-  const R a5 = d_jy * ((R)1 / (R)6), a6 = d_qy * ((R)1 / (R)12);
-  const R a7 = d_xx * (R)0.25, a8 = d_xy * (R)0.25;
-  const R ax = a0 - a1 - (R)2 * a2;  // common to i = 1..4
-  const R dg = a0 + (R)2 * a1 + a2;  // common to i = 5..8
-  g[0] -= a0 + (R)4 * (a2 - a1);
-  g[1] -= ax + a3 - (R)2 * a4 + a7;
-  g[2] -= ax + a5 - (R)2 * a6 - a7;
-  g[3] -= ax - a3 + (R)2 * a4 + a7;
-  g[4] -= ax - a5 + (R)2 * a6 - a7;
-  const R p34 = a3 + a4, p56 = a5 + a6;
-  g[5] -= dg + p34 + p56 + a8;
-  g[6] -= dg - p34 + p56 - a8;
-  g[7] -= dg - p34 - p56 + a8;
-  g[8] -= dg + p34 - p56 - a8;
-}
-
-template <typename R>
-__device__ __forceinline__ void collide_mrt5(const SpParams &P, const Macro<R> &m, R g[5]) {
-  // D2Q5 moments (1, c_x, c_y, 5|c|^2 - 4c^2, c_x^2 - c_y^2) scaled by c^-n; rates
-  // (0, 1/tau_T, 1/tau_T, 1/dt, 1/dt); source Delta t (I - dt Lambda/2) M (w qdot).
-  const R ic = K<R>(P).inv_c, dt = K<R>(P).dt;
-  const R dT = m.T - K<R>(P).T0;
-  const R m1 = g[1] - g[3], m2 = g[2] - g[4];
-  const R m3 = -(R)4 * g[0] + ((g[1] + g[2]) + (g[3] + g[4]));
-  const R m4 = (g[1] + g[3]) - (g[2] + g[4]);
-  const R sT = K<R>(P).omegaT;
-  const R d0 = -dt * m.qd;
-  const R d1 = sT * (m1 - m.T * m.ux * ic);
-  const R d2 = sT * (m2 - m.T * m.uy * ic);
-  // e-moment: rate 1/dt, equilibrium -(2/3) dT, source -(2/3) qdot with factor 1/2
-  const R d3 = (m3 + (R)(2.0 / 3.0) * dT) - K<R>(P).hdt * (-(R)(2.0 / 3.0) * m.qd);
-  const R d4 = m4;
-  const R a0 = d0 * (R)0.2, a1 = d1 * (R)0.5, a2 = d2 * (R)0.5, a3 = d3 * (R)0.05, a4 = d4 * (R)0.25;
-  g[0] -= a0 - (R)4 * a3;
-  g[1] -= a0 + a1 + a3 + a4;
-  g[2] -= a0 + a2 + a3 - a4;
-  g[3] -= a0 - a1 + a3 + a4;
-  g[4] -= a0 - a2 + a3 - a4;
+  const SpConst<R> &k = K<R>(P);
+  const R d13 = g[1] - g[3], d24 = g[2] - g[4], d57 = g[5] - g[7], d68 = g[6] - g[8];
+  const R a13 = g[1] + g[3], a24 = g[2] + g[4], a57 = g[5] + g[7], a68 = g[6] + g[8];
+  const R S = P.qdot ? m.sumg + k.dt * m.qd : m.sumg;
+  const R p9 = S * ((R)1 / (R)9), p36 = S * ((R)1 / (R)36);
+  const R tx = d57 - d68, ty = d57 + d68;  // the diagonals' share of the first moment
+  const R ex = off_eq(m, k.T0, d13 + tx, m.hx), ey = off_eq(m, k.T0, d24 + ty, m.hy);
+  const R ox = ((R)2 * tx - d13) * ((R)1 / (R)6) - k.q1T * ex, oy = ((R)2 * ty - d24) * ((R)1 / (R)6) - k.q1T * ey;
+  const R w = (R)0.5 * (ox + oy) + k.q2T * (ex + ey), v = (R)0.5 * (oy - ox) + k.q2T * (ey - ex);
+  const R p13 = p9 - (R)0.5 * a13, p24 = p9 - (R)0.5 * a24, p57 = p36 - (R)0.5 * a57, p68 = p36 - (R)0.5 * a68;
+  g[0] = S - (R)4 * (p9 + p36);
+  g[1] += p13 + ox;
+  g[3] += p13 - ox;
+  g[2] += p24 + oy;
+  g[4] += p24 - oy;
+  g[5] += p57 - w;
+  g[7] += p57 + w;
+  g[6] += p68 - v;
+  g[8] += p68 + v;
 }
 
 template <typename R, int FLOW, int TH>
 __device__ __forceinline__ void collide(const SpParams &P, const Macro<R> &m, R f[9], R *g) {
-  if (FLOW == FLOW_BGK) collide_bgk9<R>(P, m, f);
-  if (FLOW == FLOW_MRT) collide_mrt9<R>(P, m, f);
-  if (TH == TH_BGK) collide_bgk5<R, 5>(P, m, g);
+  if (FLOW != FLOW_NONE) collide_flow<R>(P, m, f);
+  if (TH == TH_BGK) collide_bgk_T<R, 5>(P, m, g);
   if (TH == TH_MRT) collide_mrt5<R>(P, m, g);
-  if (TH == TH_BGK9) collide_bgk5<R, 9>(P, m, g);
+  if (TH == TH_BGK9) collide_bgk_T<R, 9>(P, m, g);
   if (TH == TH_MRT9) collide_mrt9T<R>(P, m, g);
 }
-
-// Dispatch of a launcher body over the supported (precision, momentum operator,
-// thermal operator) combinations; CALL(PREC, FLOW, TH) names one instantiation.
-#define LBM_SP_DISPATCH(PREC_, FLOW_, TH_, CALL)                                      \
-  do {                                                                                \
-    if (PREC_ == 0) {                                                                 \
-      if (FLOW_ == FLOW_BGK && TH_ == TH_NONE) { CALL(0, FLOW_BGK, TH_NONE); }        \
-      else if (FLOW_ == FLOW_BGK && TH_ == TH_BGK) { CALL(0, FLOW_BGK, TH_BGK); }     \
-      else if (FLOW_ == FLOW_BGK && TH_ == TH_MRT) { CALL(0, FLOW_BGK, TH_MRT); }     \
-      else if (FLOW_ == FLOW_MRT && TH_ == TH_NONE) { CALL(0, FLOW_MRT, TH_NONE); }   \
-      else if (FLOW_ == FLOW_MRT && TH_ == TH_BGK) { CALL(0, FLOW_MRT, TH_BGK); }     \
-      else if (FLOW_ == FLOW_MRT && TH_ == TH_MRT) { CALL(0, FLOW_MRT, TH_MRT); }     \
-      else if (FLOW_ == FLOW_NONE && TH_ == TH_BGK) { CALL(0, FLOW_NONE, TH_BGK); }   \
-      else if (FLOW_ == FLOW_NONE && TH_ == TH_MRT) { CALL(0, FLOW_NONE, TH_MRT); }   \
-      else if (FLOW_ == FLOW_BGK && TH_ == TH_BGK9) { CALL(0, FLOW_BGK, TH_BGK9); }   \
-      else if (FLOW_ == FLOW_BGK && TH_ == TH_MRT9) { CALL(0, FLOW_BGK, TH_MRT9); }   \
-      else if (FLOW_ == FLOW_MRT && TH_ == TH_BGK9) { CALL(0, FLOW_MRT, TH_BGK9); }   \
-      else if (FLOW_ == FLOW_MRT && TH_ == TH_MRT9) { CALL(0, FLOW_MRT, TH_MRT9); }   \
-      else return cudaErrorInvalidValue;                                              \
-    } else {                                                                          \
-      if (FLOW_ == FLOW_BGK && TH_ == TH_NONE) { CALL(1, FLOW_BGK, TH_NONE); }        \
-      else if (FLOW_ == FLOW_BGK && TH_ == TH_BGK) { CALL(1, FLOW_BGK, TH_BGK); }     \
-      else if (FLOW_ == FLOW_BGK && TH_ == TH_MRT) { CALL(1, FLOW_BGK, TH_MRT); }     \
-      else if (FLOW_ == FLOW_MRT && TH_ == TH_NONE) { CALL(1, FLOW_MRT, TH_NONE); }   \
-      else if (FLOW_ == FLOW_MRT && TH_ == TH_BGK) { CALL(1, FLOW_MRT, TH_BGK); }     \
-      else if (FLOW_ == FLOW_MRT && TH_ == TH_MRT) { CALL(1, FLOW_MRT, TH_MRT); }     \
-      else if (FLOW_ == FLOW_NONE && TH_ == TH_BGK) { CALL(1, FLOW_NONE, TH_BGK); }   \
-      else if (FLOW_ == FLOW_NONE && TH_ == TH_MRT) { CALL(1, FLOW_NONE, TH_MRT); }   \
-      else if (FLOW_ == FLOW_BGK && TH_ == TH_BGK9) { CALL(1, FLOW_BGK, TH_BGK9); }   \
-      else if (FLOW_ == FLOW_BGK && TH_ == TH_MRT9) { CALL(1, FLOW_BGK, TH_MRT9); }   \
-      else if (FLOW_ == FLOW_MRT && TH_ == TH_BGK9) { CALL(1, FLOW_MRT, TH_BGK9); }   \
-      else if (FLOW_ == FLOW_MRT && TH_ == TH_MRT9) { CALL(1, FLOW_MRT, TH_MRT9); }   \
-      else return cudaErrorInvalidValue;                                              \
-    }                                                                                 \
-  } while (0)
 
 }  // namespace lbmk

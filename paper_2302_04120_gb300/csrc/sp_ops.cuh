@@ -30,14 +30,16 @@ struct SpOps {
 };
 
 // Every supported combination, X(PREC, FLOW, TH), in four groups (one unit each).
-#define LBM_SP_COMBOS_A(X) X(0, FLOW_BGK, TH_NONE) X(0, FLOW_BGK, TH_BGK) X(0, FLOW_BGK, TH_MRT) \
-  X(0, FLOW_MRT, TH_NONE) X(0, FLOW_MRT, TH_BGK) X(0, FLOW_MRT, TH_MRT)
-#define LBM_SP_COMBOS_B(X) X(0, FLOW_NONE, TH_BGK) X(0, FLOW_NONE, TH_MRT) X(0, FLOW_BGK, TH_BGK9) \
-  X(0, FLOW_BGK, TH_MRT9) X(0, FLOW_MRT, TH_BGK9) X(0, FLOW_MRT, TH_MRT9)
-#define LBM_SP_COMBOS_C(X) X(1, FLOW_BGK, TH_NONE) X(1, FLOW_BGK, TH_BGK) X(1, FLOW_BGK, TH_MRT) \
-  X(1, FLOW_MRT, TH_NONE) X(1, FLOW_MRT, TH_BGK) X(1, FLOW_MRT, TH_MRT)
-#define LBM_SP_COMBOS_D(X) X(1, FLOW_NONE, TH_BGK) X(1, FLOW_NONE, TH_MRT) X(1, FLOW_BGK, TH_BGK9) \
-  X(1, FLOW_BGK, TH_MRT9) X(1, FLOW_MRT, TH_BGK9) X(1, FLOW_MRT, TH_MRT9)
+// Momentum BGK runs in the FLOW_MRT kernels (all rates dt / tau, see collide_flow).
+#define LBM_SP_COMBOS_A(X) X(0, FLOW_MRT, TH_NONE) X(0, FLOW_MRT, TH_BGK) X(0, FLOW_MRT, TH_MRT)
+#define LBM_SP_COMBOS_B(X) X(0, FLOW_NONE, TH_BGK) X(0, FLOW_NONE, TH_MRT) X(0, FLOW_MRT, TH_BGK9) X(0, FLOW_MRT, TH_MRT9)
+#define LBM_SP_COMBOS_C(X) X(1, FLOW_MRT, TH_NONE) X(1, FLOW_MRT, TH_BGK) X(1, FLOW_MRT, TH_MRT)
+#define LBM_SP_COMBOS_D(X) X(1, FLOW_NONE, TH_BGK) X(1, FLOW_NONE, TH_MRT) X(1, FLOW_MRT, TH_BGK9) X(1, FLOW_MRT, TH_MRT9)
 #define LBM_SP_COMBOS(X) LBM_SP_COMBOS_A(X) LBM_SP_COMBOS_B(X) LBM_SP_COMBOS_C(X) LBM_SP_COMBOS_D(X)
+
+// Dispatch over the combinations inside a function with int prec, flow, th: BODY(PREC,
+// FLOW, TH) names one instantiation and returns.
+#define LBM_SP_CASE(A, B, C) \
+  if (prec == A && flow == B && th == C) LBM_SP_BODY(A, B, C);
 
 }  // namespace lbmk

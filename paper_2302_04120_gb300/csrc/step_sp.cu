@@ -43,48 +43,47 @@ namespace lbmk {
 static dim3 grid_for(int nx, int ny, dim3 b) { return dim3((nx + b.x - 1) / b.x, (ny + b.y - 1) / b.y); }
 
 cudaError_t sp_step(const SpParams &P, int prec, int flow, int th, dim3 block, cudaStream_t s) {
-#define CALL(A, B, C) return SpOps<A, B, C>::step(P, block, s)
-  LBM_SP_DISPATCH(prec, flow, th, CALL);
-#undef CALL
+#define LBM_SP_BODY(A, B, C) return SpOps<A, B, C>::step(P, block, s)
+  LBM_SP_COMBOS(LBM_SP_CASE)
+#undef LBM_SP_BODY
   return cudaErrorInvalidValue;
 }
 
 cudaError_t sp_step_occ(const SpParams &P, int prec, int flow, int th, dim3 block, cudaStream_t s) {
-#define CALL(A, B, C) return SpOps<A, B, C>::step_occ(P, block, s)
-  LBM_SP_DISPATCH(prec, flow, th, CALL);
-#undef CALL
+#define LBM_SP_BODY(A, B, C) return SpOps<A, B, C>::step_occ(P, block, s)
+  LBM_SP_COMBOS(LBM_SP_CASE)
+#undef LBM_SP_BODY
   return cudaErrorInvalidValue;
 }
 
 cudaError_t sp_batch_step(const SpParams *table, const int4 *tiles, int ntiles, int prec, int flow, int th, dim3 block,
                           int grid, cudaStream_t s) {
-#define CALL(A, B, C) return SpOps<A, B, C>::batch(table, tiles, ntiles, block, grid, s)
-  LBM_SP_DISPATCH(prec, flow, th, CALL);
-#undef CALL
+#define LBM_SP_BODY(A, B, C) return SpOps<A, B, C>::batch(table, tiles, ntiles, block, grid, s)
+  LBM_SP_COMBOS(LBM_SP_CASE)
+#undef LBM_SP_BODY
   return cudaErrorInvalidValue;
 }
 
 int sp_batch_occupancy(int prec, int flow, int th, int threads) {
-#define CALL(A, B, C) \
-  if (prec == A && flow == B && th == C) return SpOps<A, B, C>::occupancy(threads);
-  LBM_SP_COMBOS(CALL)
-#undef CALL
+#define LBM_SP_BODY(A, B, C) return SpOps<A, B, C>::occupancy(threads)
+  LBM_SP_COMBOS(LBM_SP_CASE)
+#undef LBM_SP_BODY
   return 0;
 }
 
 cudaError_t sp_init(const SpParams &P, int prec, int flow, int th, const double *a, const double *ux,
                     const double *uy, const double *b, dim3 block, cudaStream_t s) {
-#define CALL(A, B, C) return SpOps<A, B, C>::init(P, a, ux, uy, b, block, s)
-  LBM_SP_DISPATCH(prec, flow, th, CALL);
-#undef CALL
+#define LBM_SP_BODY(A, B, C) return SpOps<A, B, C>::init(P, a, ux, uy, b, block, s)
+  LBM_SP_COMBOS(LBM_SP_CASE)
+#undef LBM_SP_BODY
   return cudaErrorInvalidValue;
 }
 
 cudaError_t sp_moments(const SpParams &P, int prec, int flow, int th, unsigned mask, double *out,
                        cudaStream_t s) {
-#define CALL(A, B, C) return SpOps<A, B, C>::moments(P, mask, out, s)
-  LBM_SP_DISPATCH(prec, flow, th, CALL);
-#undef CALL
+#define LBM_SP_BODY(A, B, C) return SpOps<A, B, C>::moments(P, mask, out, s)
+  LBM_SP_COMBOS(LBM_SP_CASE)
+#undef LBM_SP_BODY
   return cudaErrorInvalidValue;
 }
 
@@ -99,9 +98,9 @@ cudaError_t sp_integrals(const SpParams &P, int prec, int flow, int th, double *
   int steps, fy;
   dim3 grid = integral_grid(P.nx, P.ny, &steps, &fy);
   if ((int)(grid.x * grid.y) > max_blocks) return cudaErrorInvalidValue;
-#define CALL(A, B, C) return SpOps<A, B, C>::integrals(P, partials, out4, counter, s)
-  LBM_SP_DISPATCH(prec, flow, th, CALL);
-#undef CALL
+#define LBM_SP_BODY(A, B, C) return SpOps<A, B, C>::integrals(P, partials, out4, counter, s)
+  LBM_SP_COMBOS(LBM_SP_CASE)
+#undef LBM_SP_BODY
   return cudaErrorInvalidValue;
 }
 

@@ -49,24 +49,23 @@ int sp_tma_encode(void *base, int pitch, int ny, int nq, int elem, int ty, CUten
 cudaError_t sp_step_tma(const SpParams &P, const CUtensorMap &map, int prec, int flow, int th, int ty, int stages,
                         int grid, int *flag, unsigned long long wait_ns, int expire_probe, cudaStream_t s) {
   if (stages < 1 || stages > kMaxStages || grid < 1 || P.local) return cudaErrorInvalidValue;
-#define CALL(A, B, C) return TmaOps<A, B, C>::step(P, map, ty, stages, grid, flag, wait_ns, expire_probe, s)
-  LBM_SP_DISPATCH(prec, flow, th, CALL);
-#undef CALL
+#define LBM_SP_BODY(A, B, C) return TmaOps<A, B, C>::step(P, map, ty, stages, grid, flag, wait_ns, expire_probe, s)
+  LBM_SP_COMBOS(LBM_SP_CASE)
+#undef LBM_SP_BODY
   return cudaErrorInvalidValue;
 }
 
 cudaError_t sp_tma_prepare(int prec, int flow, int th) {
-#define CALL(A, B, C) return TmaOps<A, B, C>::prepare()
-  LBM_SP_DISPATCH(prec, flow, th, CALL);
-#undef CALL
+#define LBM_SP_BODY(A, B, C) return TmaOps<A, B, C>::prepare()
+  LBM_SP_COMBOS(LBM_SP_CASE)
+#undef LBM_SP_BODY
   return cudaErrorInvalidValue;
 }
 
 int sp_tma_occupancy(int prec, int flow, int th, int ty, int stages) {
-#define CALL(A, B, C) \
-  if (prec == A && flow == B && th == C) return TmaOps<A, B, C>::occupancy(ty, stages);
-  LBM_SP_COMBOS(CALL)
-#undef CALL
+#define LBM_SP_BODY(A, B, C) return TmaOps<A, B, C>::occupancy(ty, stages)
+  LBM_SP_COMBOS(LBM_SP_CASE)
+#undef LBM_SP_BODY
   return 0;
 }
 
