@@ -255,8 +255,8 @@ lbm_status lbm_set_wait_limit(lbm_t h, double seconds, int expire_next);
  * of 32..256 threads and TMA-staged persistent launches, see lbm_set_launch) on the
  * next step, without advancing the solution (the timed launches repeat that step into
  * the same destination).  out_block (may be NULL) receives the chosen thread-block
- * shape {block_x, block_y}.  Single-phase solves only; the default is a 64 x 4 grid
- * launch.
+ * shape {block_x, block_y}.  Single-phase solves only; the default is a grid launch
+ * (reported as 64 x 4) whose block shape the library takes by grid size.
  * Errors: LBM_ERR_STATE (not initialised), LBM_ERR_ARG, LBM_ERR_CUDA.
  */
 lbm_status lbm_autotune(lbm_t h, int out_block[2]);
@@ -276,7 +276,8 @@ lbm_status lbm_probe_fma_rate(int precision, double *gflops);
  * Launch configuration of the single-phase step (no counterpart in the paper: a
  * choice of memory pipeline for the same arithmetic).  cfg[4]:
  *  {LBM_LAUNCH_GRID, block_x, block_y, 0}: one thread per node, block_x a multiple
- *     of 32, block_x * block_y <= 256 (the default, 64 x 4);
+ *     of 32, block_x * block_y <= 256 (the default, 64 x 4: until a launch is set here
+ *     or by lbm_autotune, the library takes the block shape and the build by grid size);
  *  {LBM_LAUNCH_GRID_OCC, block_x, block_y, 0}: the same kernel built for more
  *     resident blocks per SM (FP32 with a thermal lattice: 6 blocks of 256 threads at
  *     40 registers instead of 4 at 64; faster on large grids, slower on short

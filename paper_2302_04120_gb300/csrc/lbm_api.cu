@@ -53,6 +53,7 @@ struct lbm_s {
   // single-phase step launch: LBM_LAUNCH_GRID (one node per thread, `block`) or
   // LBM_LAUNCH_TMA (persistent CTAs of 32 x tma_ty threads, boxes staged by TMA)
   int launch_kind;
+  int launch_set;  // chosen by lbm_set_launch / lbm_autotune; 0: by size, see step_launch
   int tma_ty, tma_stages, tma_ctas;  // tma_ctas: CTAs per SM
   unsigned long long tma_wait_ns;    // wall-time limit of each staged-copy wait
   int tma_expire_next;               // self-test: the next TMA-staged step's waits run out
@@ -75,7 +76,7 @@ struct lbm_s {
 // Everything a run of grid-launched steps depends on besides device memory contents:
 // the kernel choice and the parameter blocks of both buffer parities.
 struct StepKey {
-  int two_phase, prec, flow, th, kind;
+  int two_phase, prec, flow, th, occ;
   dim3 block;
   double sink_conv, sink_Tinf;
   lbmk::MpParams mp[2];
@@ -633,14 +634,62 @@ static cudaError_t sink_refresh(const lbm_t h, int from, int pre, cudaStream_t s
                            p.precision, st);
 }
 
+// Block shape and build of the single-phase grid launch.  As set by the caller, or by
+// size while nothing was set (measured on GB300, back-to-back steps, us per step):
+//  * one-warp blocks while all of them are resident at once (64 registers: 32 warps per
+//    SM in FP32; 80: 24 in FP64): the boundary frame's warps, the longest, then spread
+//    over the SMs.  FP32 1024 x 128: 8.0 with 64 x 4 blocks, 4.2 with 32 x 1; FP64 64 x 33
+//    BGK: 8.5 and 5.3;
+//  * above that blocks of two warps in FP32 (2048 x 256: 9.2 with 64 x 4, 6.8 with 64 x 1,
+//    9.5 with 32 x 1, whose 32 blocks per SM leave registers unused) and of four in FP64
+//    (1024 x 128: 30.1, 26.7);
+//  * FP32 with a D2Q5 thermal lattice whose two state buffers exceed the 129 MB L2: the
+//    build for 6 resident blocks per SM with 256 x 1 blocks (8192 x 4096: 545 against 555
+//    with 64 x 1 and 580 with 64 x 4; on the D2Q9 lattice it is slower: 727 against 704).
+// Wide shapes only where the last block of a row wastes little; the shape reported by
+// lbm_launch_config stays the nominal one.
+struct StepLaunch {
+  int occ;  // the build for more resident blocks
+  dim3 block;
+};
+
+static StepLaunch step_launch(const lbm_t h) {
+  StepLaunch l = {h->launch_kind == LBM_LAUNCH_GRID_OCC, h->block};
+  if (h->launch_set || h->launch_kind == LBM_LAUNCH_TMA) return l;
+  const long long nodes = (long long)h->p.nx * h->p.ny;
+  const int fp64 = h->p.precision == LBM_FP64;
+  dim3 b;
+  int occ = 0;
+  if (nodes <= 32ll * h->nsm * (fp64 ? 24 : 32)) {
+    b = dim3(32, 1);
+  } else if (!fp64 && h->p.thermal == LBM_D2Q5 && h->p.flow && 2.0 * h->nq * h->plane * h->elem > 129e6) {
+    b = dim3(256, 1);
+    occ = 1;
+  } else {
+    const int t = fp64 ? 128 : 64;
+    b = h->p.nx >= 1024 || h->p.nx % t == 0 ? dim3(t, 1) : dim3(32, t / 32);
+  }
+  // rows of blocks, the frame's included, within the grid's limit; else the nominal shape
+  const long long gx = (h->p.nx + b.x - 1) / b.x, nt = b.x * b.y;
+  const long long frame = (lbmk::frame_nodes(h->p.nx, h->p.ny) + nt - 1) / nt;
+  if ((h->p.ny + b.y - 1) / b.y + (frame + gx - 1) / gx > 65535) return l;
+  l.occ = occ;
+  l.block = b;
+  return l;
+}
+
+static cudaError_t sp_launch(const lbm_t h, const SpParams &P, int flow, int th, cudaStream_t st) {
+  const StepLaunch l = step_launch(h);
+  return l.occ ? lbmk::sp_step_occ(P, h->p.precision, flow, th, l.block, st)
+               : lbmk::sp_step(P, h->p.precision, flow, th, l.block, st);
+}
+
 // One grid-launched step reading buffer `from` (two-phase or single phase).
 static cudaError_t launch_grid_step(const lbm_t h, int from, int flow, int th, cudaStream_t st) {
   if (two_phase(h)) return lbmk::mp_step(mp_params(h, from), h->p.precision, st);
   const cudaError_t e = sink_refresh(h, from, 0, st);
   if (e != cudaSuccess) return e;
-  if (h->launch_kind == LBM_LAUNCH_GRID_OCC)
-    return lbmk::sp_step_occ(sp_params(h, from), h->p.precision, flow, th, h->block, st);
-  return lbmk::sp_step(sp_params(h, from), h->p.precision, flow, th, h->block, st);
+  return sp_launch(h, sp_params(h, from), flow, th, st);
 }
 
 static void step_key(const lbm_t h, int flow, int th, StepKey *k) {
@@ -649,8 +698,9 @@ static void step_key(const lbm_t h, int flow, int th, StepKey *k) {
   k->prec = h->p.precision;
   k->flow = flow;
   k->th = th;
-  k->kind = h->launch_kind;
-  k->block = h->block;
+  const StepLaunch l = step_launch(h);
+  k->occ = l.occ;
+  k->block = l.block;
   k->sink_conv = h->sink_conv;
   k->sink_Tinf = h->sink_Tinf;
   for (int b = 0; b < 2; b++) {
@@ -720,9 +770,7 @@ static lbm_status advance(lbm_t h, long n) {
                             h->nsm * h->tma_ctas, step_flag(h), h->tma_wait_ns, h->tma_expire_next, h->stream);
       h->tma_expire_next = 0;
     } else {
-      SpParams P = sp_params(h, h->cur);
-      e = h->launch_kind == LBM_LAUNCH_GRID_OCC ? lbmk::sp_step_occ(P, h->p.precision, flow, th, h->block, h->stream)
-                                             : lbmk::sp_step(P, h->p.precision, flow, th, h->block, h->stream);
+      e = sp_launch(h, sp_params(h, h->cur), flow, th, h->stream);
     }
     if (e != cudaSuccess) return fail(h, LBM_ERR_CUDA, "step launch: %s", cudaGetErrorString(e));
     h->cur = 1 - h->cur;
@@ -1280,7 +1328,7 @@ extern "C" lbm_status lbm_adjoint(lbm_t h, long steps, int ckpt_every, const dou
         Q.local = (m == 0 && k == 1) ? 1 : 0;
         Q.src = (char *)seg + sbytes * (size_t)(k - 1);
         Q.dst = (char *)seg + sbytes * (size_t)k;
-        ACU(lbmk::sp_step(Q, p.precision, lbmk::FLOW_MRT, lbmk::TH_MRT, h->block, h->stream));
+        ACU(sp_launch(h, Q, lbmk::FLOW_MRT, lbmk::TH_MRT, h->stream));
       }
       for (long t = s1; t >= s0; t--) {
         const long k = t - s0 + 1;
@@ -1386,6 +1434,7 @@ static lbm_status check_launch(lbm_t h, const int cfg[4]) {
 
 static void apply_launch(lbm_t h, const int cfg[4]) {
   h->launch_kind = cfg[0];
+  h->launch_set = 1;
   if (cfg[0] != LBM_LAUNCH_TMA) {
     h->block = dim3(cfg[1], cfg[2]);
   } else {
