@@ -230,13 +230,29 @@ static SpParams sp_params(const lbm_t h, int from_buf) {
 
 template <typename R>
 static void fill_mp_const(const lbmk::MpParams &P, lbmk::MpConst<R> &k) {
-  k.c = (R)P.c; k.dt = (R)P.dt; k.inv_cs2 = (R)P.inv_cs2; k.g3 = (R)P.g3; k.l6 = (R)P.l6;
-  k.beta = (R)P.beta; k.kappa = (R)P.kappa; k.rho_g = (R)P.rho_g; k.drl = (R)(P.rho_l - P.rho_g);
-  k.nu_g = (R)P.nu_g; k.dnu = (R)(P.nu_l - P.nu_g); k.zg = (R)(P.rho_g * P.nu_g);
-  k.dzeta = (R)(P.rho_l * P.nu_l - P.rho_g * P.nu_g); k.inv_cs2dt = (R)P.inv_cs2dt;
-  k.Fx = (R)P.Fx; k.Fy = (R)P.Fy; k.hdt = (R)(0.5 * P.dt); k.pcoef = (R)(P.cs2 * 1.8);
-  k.om_h = (R)P.om_h; k.sfac_h = (R)P.sfac_h; k.aint_coef = (R)P.aint_coef; k.inv_dt = (R)P.inv_dt;
-  k.ic = (R)1 / (R)P.c;
+  const double drl = P.rho_l - P.rho_g, hdt_ic = 0.5 * P.dt / P.c;
+  const double g = 3.0 / P.dx / 36.0, l = 6.0 / (P.dx * P.dx) / 36.0;  // Eqs. gradient, laplacian
+  const double inv_cs2dt = 1.0 / (P.cs2 * P.dt), om = P.dt / P.tauphi;
+  const double sfac = (1.0 - 0.5 * om) * P.dt / (2.0 * P.c);           // Eq. source_term_interface
+  k.c = (R)P.c;
+  k.rho_g = (R)P.rho_g;
+  k.rho_g_lo = (R)(P.rho_g - (double)k.rho_g);
+  k.drl = (R)drl;
+  k.drl_lo = (R)(drl - (double)k.drl);
+  k.hdt_ic = (R)hdt_ic;
+  k.Fx = (R)P.Fx;
+  k.Fy = (R)P.Fy;
+  k.kb = (R)(4.0 * P.beta * hdt_ic * g);
+  k.kl = (R)(P.kappa * l * hdt_ic * g);
+  k.kg = (R)(0.5 * P.dt * P.c * drl * g);
+  k.tau0 = (R)(P.nu_g * inv_cs2dt + 0.5);
+  k.dtau = (R)((P.nu_l - P.nu_g) * inv_cs2dt);
+  k.zg = (R)(P.rho_g * P.nu_g * inv_cs2dt);
+  k.dzeta = (R)((P.rho_l * P.nu_l - P.rho_g * P.nu_g) * inv_cs2dt);
+  k.om_h = (R)om;
+  k.hom_h = (R)(0.5 * om);
+  k.s1 = (R)(sfac / P.dt);
+  k.s2 = (R)(sfac * 4.0 * P.cs2 / P.W);
 }
 
 static lbmk::MpParams mp_params(const lbm_t h, int from_buf) {
@@ -250,14 +266,6 @@ static lbmk::MpParams mp_params(const lbm_t h, int from_buf) {
   P.beta = 12.0 * p.sigma / p.W;   // beta = 12 sigma / W
   P.W = p.W;
   P.tauphi = h->tauphi;
-  P.inv_cs2 = 1.0 / h->cs2;
-  P.g3 = 3.0 / p.dx;
-  P.l6 = 6.0 / (p.dx * p.dx);
-  P.inv_cs2dt = 1.0 / (h->cs2 * p.dt);
-  P.om_h = p.dt / h->tauphi;
-  P.sfac_h = (1.0 - p.dt / (2.0 * h->tauphi)) * p.dt;
-  P.aint_coef = 4.0 * h->cs2 / p.W;
-  P.inv_dt = 1.0 / p.dt;
   P.nu_rule = p.nu_rule;
   P.z_mrt = p.z_op == LBM_MRT;
   P.qy_literal = (p.literal & 2) ? 1 : 0;
@@ -265,6 +273,7 @@ static lbmk::MpParams mp_params(const lbm_t h, int from_buf) {
   P.ywall = h->bc[2] != LBM_BC_PERIODIC || h->bc[3] != LBM_BC_PERIODIC;
   P.Fx = p.body_force[0]; P.Fy = p.body_force[1];
   P.force = h->d_force;
+  P.forced = P.Fx != 0.0 || P.Fy != 0.0 || P.force;
   P.local = h->pre;
   P.src = h->buf[from_buf];
   P.dst = h->buf[1 - from_buf];

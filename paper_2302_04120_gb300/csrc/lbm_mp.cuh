@@ -8,8 +8,12 @@ namespace lbmk {
 // FP32 kernels convert nothing per thread on GB300's slow FP64 pipe).
 template <typename R>
 struct MpConst {
-  R c, dt, inv_cs2, g3, l6, beta, kappa, rho_g, drl, nu_g, dnu, zg, dzeta, inv_cs2dt;
-  R Fx, Fy, hdt, pcoef, om_h, sfac_h, aint_coef, inv_dt, ic;
+  R c, rho_g, rho_g_lo, drl, drl_lo;  // drl = rho_l - rho_g; _lo: what R rounds off
+  R hdt_ic, Fx, Fy;                   // dt / (2 c), body force
+  R kb, kl, kg;                       // dt / (2 c) mu grad phi and (dt / 2) c grad rho from the
+                                      // stencil sums r = 36 dx / 3 grad phi (see mp_macro)
+  R tau0, dtau, zg, dzeta;            // tau / dt = tau0 + phi dtau, or (zg + phi dzeta) / rho + 1/2
+  R om_h, hom_h, s1, s2;              // dt / tau_phi and half of it; sources of the odd h pairs
 };
 
 // Two-phase solve; each axis periodic or bounded by resting half-way walls on both
@@ -20,12 +24,10 @@ struct MpParams {
   double c, cs2, dt, dx;
   double rho_l, rho_g, nu_l, nu_g;
   double kappa, beta, W, tauphi;
-  // derived constants (host-side): 1/c_s^2, 3/dx, 6/dx^2, 1/(c_s^2 dt), dt/tau_phi,
-  // (1 - dt/(2 tau_phi)) dt, 4 c_s^2 / W, 1/dt
-  double inv_cs2, g3, l6, inv_cs2dt, om_h, sfac_h, aint_coef, inv_dt;
   int nu_rule, z_mrt, qy_literal;
   int xwall, ywall;  // 1: the axis ends at resting walls (bounce-back, mirrored phi)
   double Fx, Fy;
+  int forced;        // a body force or a force field acts
   MpConst<double> kd;
   MpConst<float> kf;
   const void *force;  // 2 planes or null

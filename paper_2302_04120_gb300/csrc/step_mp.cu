@@ -15,12 +15,22 @@
 //     [Lambda]_dim of Sec. 3, Eqs. zeq_liang, s_i_Liang,
 //     forcing_term_pressure_evolution); store h*, z* and phi u for the next
 //     explicit d_t(phi u).
+// The collisions work on pairs of opposite populations (as in sp_device.cuh): the FP64
+// form is bound by GB300's FP64 pipe, so its time is the number of FP64 instructions per
+// node; lengths, dt and c are folded into host-filled constants.
 // In the FP32 form the populations and (phi u) are stored in FP32 and the
-// collision runs in FP32, while rho(phi), u and p are recovered in FP64 across the
-// interface and in the gas (phi < 0.999): at the ~43000 density ratio of saturated
-// water u = j / rho divides by rho_g = 0.023.  In the liquid bulk FP32 resolves them.
+// collision runs in FP32, while rho(phi), u and p are recovered in pairs of floats
+// (hi + lo, about 48 bits) across the interface and in the gas (phi < 0.999): at the
+// ~43000 density ratio of saturated water u = j / rho divides by rho_g = 0.023.  In the
+// liquid bulk FP32 resolves them.  The pairs run on the FP32 pipe; the same recovery in
+// FP64 (about 60 instructions of 16 cycles a warp) held whole tiles of the gas on the
+// FP64 pipe.  Results are rounded to FP32 either way.
+// Measured before and after pairs of populations, float pairs and the narrow blocks: FP32
+// 512^2 bubble 12.9 -> 10.7 us per step, 4096^2 435 -> 390 us, error against a 64-bit
+// solution after 100 steps 6.6e-6 -> 3.5e-6; FP64 10 x 400 layered flow 15.9 -> 9.5 us.
 #include <cuda_runtime.h>
 
+#include "compensated.cuh"
 #include "lattice.cuh"
 #include "lbm_mp.cuh"
 
@@ -30,8 +40,13 @@ namespace {
 
 // Tiles are 32 nodes wide and BY = 8 rows high, or 2 rows on grids too small to give
 // every SM several 32 x 8 tiles (the FP64 collision is then spread over more SMs).
+// Grids of at most kNarrow columns (layered flow between plates, uniform along x) take
+// one-warp blocks of whole rows (BY = 0): a warp holds 32 / nx rows instead of 32 / nx
+// warps each nx lanes, and the halo is the two rows beside the block.
 constexpr int BX = 32;
 constexpr int kSmallGridBlocks = 608;  // 4 x 152 SMs: fewer 32 x 8 tiles take BY = 2
+constexpr int kNarrow = 16;
+constexpr int kNarrowTile = 104;       // (rows + 2) (nx + 2), rows = 32 / nx, nx = 1..kNarrow
 
 __device__ __forceinline__ int wrapi(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 __device__ __forceinline__ int modi(int a, int n) { int r = a % n; return r < 0 ? r + n : r; }
@@ -78,13 +93,29 @@ __device__ __forceinline__ void pull_z_at(const MpParams &P, const S *sn, R z[9]
   for (int q = 0; q < 9; q++) z[q] = (R)sn[q * P.plane - (long long)cy9(q) * P.pitch - cx9(q)];
 }
 
-// Quotient in the working precision: exact in FP64; in FP32 the approximate
-// reciprocal-based divide (about 2 ulp), which spares the IEEE divide sequence.
-__device__ __forceinline__ double qdiv(double a, double b) { return a / b; }
-__device__ __forceinline__ float qdiv(float a, float b) { return __fdividef(a, b); }
-// 1 / |g| for g2 = |g|^2 > 0, else 0 (same precision split).
-__device__ __forceinline__ double inv_norm(double g2) { return g2 != 0.0 ? 1.0 / sqrt(g2) : 0.0; }
+// 1 / x and 1 / sqrt(x) in the working precision.  FP32: the hardware approximations
+// (one unit in the last place).  FP64: from them by third-order iterations in e, e = 1 -
+// x r or 1 - x y^2 (1 / (1 - e) = 1 + e + e^2 .., 1 / sqrt(1 - e) = 1 + e / 2 + 3 e^2 / 8 ..).
+__device__ __forceinline__ float rcp(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ double rcp(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+// 1 / |g| for g2 = |g|^2 > 0, else 0.
 __device__ __forceinline__ float inv_norm(float g2) { return g2 != 0.0f ? rsqrtf(g2) : 0.0f; }
+__device__ __forceinline__ double inv_norm(double g2) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(g2));
+  const double e = fma(-g2 * y, y, 1.0);
+  y = fma(y * e, fma(e, 0.375, 0.5), y);
+  return g2 > 1e-300 ? y : 0.0;  // a smaller |g|^2 has left the normal range
+}
 
 template <typename S, typename R>
 __device__ __forceinline__ void pull_z(const MpParams &P, const S *src, int i, int j, R z[9]) {
@@ -92,203 +123,223 @@ __device__ __forceinline__ void pull_z(const MpParams &P, const S *src, int i, i
   for (int q = 0; q < 9; q++) z[q] = (R)src[pull_src(P, q, opp9(q), cx9(q), cy9(q), i, j)];
 }
 
-// Macroscopic state of a node.  The order parameter, its stencils, the chemical
-// potential, the forces and the relaxation rates are in the working precision R;
-// rho, u and p -- the recovery that divides by rho_g ~ 0.023 at the interface --
-// are in FP64 in both forms.
+// Macroscopic state of a node in the working precision.  h = u / c; j = rho h; rx, ry are
+// 36 / (3 / dx) grad phi; the half force H = dt F / (2 c) and U = (dt / 2) u . grad rho are
+// what the collision needs of F and grad rho; Pp = p / c_s^2.
 template <typename R>
 struct MpMacro {
-  R phi, mu, gx, gy, nxv, nyv, Fx, Fy, drx, dry, wb;  // wb = dt / tau
-  R rho, ux, uy, p;
+  R phi, rx, ry, rn, Hx, Hy, snu;  // snu = dt / tau
+  R rho, hx, hy, jx, jy, ru, U, Pp;
 };
 
-// Gradient/Laplacian from the shared tile, then rho, nu, tau, F, u, p.
 // Liquid nodes with phi above this use the working-precision recovery of rho, u, p;
-// all others (the interface, its tanh tails and the gas) recover in FP64.
-constexpr float kPhiFp64Below = 0.999f;
+// all others (the interface, its tanh tails and the gas) recover in float pairs.
+constexpr float kPhiFineBelow = 0.999f;
 
-template <typename R>
-__device__ __forceinline__ void mp_macro(const MpParams &P, const R (*tile)[BX + 2], int tx, int ty,
-                                         const R z[9], R fext_x, R fext_y, MpMacro<R> &m) {
-  // D2Q9 neighbours phi(x + c_i dt)
-  const R pc = tile[ty][tx];
-  const R pE = tile[ty][tx + 1], pW = tile[ty][tx - 1];
-  const R pN = tile[ty + 1][tx], pS = tile[ty - 1][tx];
-  const R pNE = tile[ty + 1][tx + 1], pNW = tile[ty + 1][tx - 1];
-  const R pSW = tile[ty - 1][tx - 1], pSE = tile[ty - 1][tx + 1];
-  // Eq. gradient: sum_i w_i c_i phi_i / (c_s^2 dt) = (3/dx) sum_i w_i e_i phi_i
-  const MpConst<R> &K = KM<R>(P);
-  const R g3 = K.g3;
-  m.gx = g3 * ((pE - pW) * ((R)1 / (R)9) + ((pNE - pNW) + (pSE - pSW)) * ((R)1 / (R)36));
-  m.gy = g3 * ((pN - pS) * ((R)1 / (R)9) + ((pNE - pSE) + (pNW - pSW)) * ((R)1 / (R)36));
-  // Eq. laplacian: sum_i 2 w_i (phi_i - phi) / (c_s^2 dt^2) = (6/dx^2) sum_i w_i (phi_i - phi)
-  const R lap = K.l6 * (((pE + pW) + (pN + pS) - (R)4 * pc) * ((R)1 / (R)9) +
-                           ((pNE + pNW) + (pSE + pSW) - (R)4 * pc) * ((R)1 / (R)36));
-  m.phi = pc;
-  // Eq. chemical_potential
-  m.mu = (R)4 * K.beta * pc * (pc - (R)1) * (pc - (R)0.5) - K.kappa * lap;
-  // normal only where |grad phi| != 0
-  const R rg = inv_norm(m.gx * m.gx + m.gy * m.gy);
-  m.nxv = m.gx * rg;
-  m.nyv = m.gy * rg;
-  const R drl = K.drl;
-  R nu;
-  if (P.nu_rule == 0) nu = K.nu_g + pc * K.dnu;
-  else nu = qdiv(K.zg + pc * K.dzeta, K.rho_g + pc * drl);
-  // tau / dt = nu / (c_s^2 dt) + 1/2 (Eq. eq_kinematic_viscosity)
-  m.wb = qdiv((R)1, nu * K.inv_cs2dt + (R)0.5);
-  m.drx = drl * m.gx;
-  m.dry = drl * m.gy;
-  m.Fx = m.mu * m.gx + K.Fx + fext_x;
-  m.Fy = m.mu * m.gy + K.Fy + fext_y;
-  // recovery of rho(phi), Eq. u_Liang, then Eq. p_Liang (u first)
-  if (sizeof(R) == 8 || pc < (R)kPhiFp64Below) {
-    // FP64 across the interface and in the gas, where u = j / rho divides by rho_g
-    double zd[9];
-#pragma unroll
-    for (int q = 0; q < 9; q++) zd[q] = (double)z[q];
-    const double c = P.c;
-    const double jx = c * ((zd[1] - zd[3]) + (zd[5] - zd[6]) + (zd[8] - zd[7]));
-    const double jy = c * ((zd[2] - zd[4]) + (zd[5] - zd[8]) + (zd[6] - zd[7]));
-    const double znz = ((zd[1] + zd[2]) + (zd[3] + zd[4])) + ((zd[5] + zd[6]) + (zd[7] + zd[8]));
-    const double rho = P.rho_g + (double)pc * (P.rho_l - P.rho_g);
-    const double inv = 1.0 / rho;
-    const double ux = (jx + 0.5 * P.dt * (double)m.Fx) * inv;
-    const double uy = (jy + 0.5 * P.dt * (double)m.Fy) * inv;
-    const double usq = ux * ux + uy * uy;
-    const double s0 = (4.0 / 9.0) * (-0.5 * usq * P.inv_cs2);  // s_0(u), Eq. s_i_Liang
-    m.rho = (R)rho;
-    m.ux = (R)ux;
-    m.uy = (R)uy;
-    m.p = (R)(P.cs2 * 1.8 * (znz + 0.5 * P.dt * (ux * (double)m.drx + uy * (double)m.dry) + rho * s0));
-  } else {
-    // liquid (rho within 0.1 % of rho_l): the working precision resolves u and p
-    const R c = K.c;
-    const R jx = c * ((z[1] - z[3]) + (z[5] - z[6]) + (z[8] - z[7]));
-    const R jy = c * ((z[2] - z[4]) + (z[5] - z[8]) + (z[6] - z[7]));
-    const R znz = ((z[1] + z[2]) + (z[3] + z[4])) + ((z[5] + z[6]) + (z[7] + z[8]));
-    const R rho = K.rho_g + pc * K.drl;
-    const R inv = qdiv((R)1, rho);
-    const R hdt = K.hdt;
-    const R ux = (jx + hdt * m.Fx) * inv, uy = (jy + hdt * m.Fy) * inv;
-    const R s0 = (R)(4.0 / 9.0) * ((R)-0.5 * (ux * ux + uy * uy) * K.inv_cs2);
-    m.rho = rho;
-    m.ux = ux;
-    m.uy = uy;
-    m.p = K.pcoef * (znz + hdt * (ux * m.drx + uy * m.dry) + rho * s0);
+// Sums of floats with the rounding errors carried along, s + e.
+struct Pair {
+  float s, e;
+  __device__ __forceinline__ void add(float x) {
+    float r;
+    two_sum(s, x, s, r);
+    e += r;
   }
+  // exact product added
+  __device__ __forceinline__ void add_product(float a, float b) {
+    const float p = __fmul_rn(a, b);  // (not contracted into the sum)
+    e += fmaf(a, b, -p);
+    add(p);
+  }
+  __device__ __forceinline__ void renorm() {
+    float r;
+    two_sum(s, e, s, r);
+    e = r;
+  }
+};
+
+// rho, u and p of Eqs. u_Liang and p_Liang (u first).  jz and znz: lattice-scaled first
+// moment and sum of z_1..8.
+__device__ __forceinline__ void recover(const MpParams &P, const double z[9], MpMacro<double> &m, double Gx, double Gy) {
+  const MpConst<double> &K = P.kd;
+  const double tx = (z[5] - z[7]) - (z[6] - z[8]), ty = (z[5] - z[7]) + (z[6] - z[8]);
+  m.rho = K.rho_g + m.phi * K.drl;
+  const double inv = rcp(m.rho);
+  m.jx = ((z[1] - z[3]) + tx) + m.Hx;
+  m.jy = ((z[2] - z[4]) + ty) + m.Hy;
+  m.hx = m.jx * inv;
+  m.hy = m.jy * inv;
+  m.ru = m.jx * m.hx + m.jy * m.hy;
+  m.U = m.hx * Gx + m.hy * Gy;
+  const double znz = ((z[1] + z[3]) + (z[2] + z[4])) + ((z[5] + z[7]) + (z[6] + z[8]));
+  m.Pp = 1.8 * ((znz + m.U) - (2.0 / 3.0) * m.ru);
+}
+
+__device__ __forceinline__ void recover(const MpParams &P, const float z[9], MpMacro<float> &m, float Gx, float Gy) {
+  const MpConst<float> &K = P.kf;
+  if (m.phi < kPhiFineBelow) {
+    Pair jx = {z[1], 0.0f}, jy = {z[2], 0.0f}, n = {z[1], 0.0f}, rho = {K.rho_g, K.rho_g_lo};
+    jx.add(-z[3]); jx.add(z[5]); jx.add(-z[7]); jx.add(-z[6]); jx.add(z[8]); jx.add(m.Hx);
+    jy.add(-z[4]); jy.add(z[5]); jy.add(-z[7]); jy.add(z[6]); jy.add(-z[8]); jy.add(m.Hy);
+    n.add(z[3]); n.add(z[2]); n.add(z[4]); n.add(z[5]); n.add(z[7]); n.add(z[6]); n.add(z[8]);
+    rho.add_product(m.phi, K.drl);
+    rho.e = fmaf(m.phi, K.drl_lo, rho.e);
+    jx.renorm();
+    jy.renorm();
+    rho.renorm();
+    float inv = rcp(rho.s);
+    inv = fmaf(inv, fmaf(-rho.s, inv, 1.0f), inv);
+    // h = j / rho: quotient of the leading parts and its remainder
+    Pair hx = {__fmul_rn(jx.s, inv), 0.0f}, hy = {__fmul_rn(jy.s, inv), 0.0f};
+    hx.e = inv * (fmaf(-hx.s, rho.s, jx.s) + fmaf(-hx.s, rho.e, jx.e));
+    hy.e = inv * (fmaf(-hy.s, rho.s, jy.s) + fmaf(-hy.s, rho.e, jy.e));
+    hx.renorm();
+    hy.renorm();
+    Pair ru = {0.0f, 0.0f}, U = {0.0f, 0.0f};
+    ru.add_product(jx.s, hx.s);
+    ru.add_product(jy.s, hy.s);
+    ru.e += jx.s * hx.e + jx.e * hx.s + jy.s * hy.e + jy.e * hy.s;
+    U.add_product(hx.s, Gx);
+    U.add_product(hy.s, Gy);
+    U.e += hx.e * Gx + hy.e * Gy;
+    ru.renorm();
+    U.renorm();
+    // znz + U - (2/3) ru, then 1.8 times that, the constants as hi + lo
+    constexpr float k23 = (float)(2.0 / 3.0), k23l = (float)(2.0 / 3.0 - (double)k23);
+    constexpr float k18 = 1.8f, k18l = (float)(1.8 - (double)k18);
+    n.add(U.s);
+    n.add_product(ru.s, -k23);
+    n.e += U.e - (ru.e * k23 + ru.s * k23l);
+    n.renorm();
+    m.rho = rho.s;
+    m.jx = jx.s;
+    m.jy = jy.s;
+    m.hx = hx.s;
+    m.hy = hy.s;
+    m.ru = ru.s;
+    m.U = U.s;
+    m.Pp = fmaf(k18, n.s, fmaf(k18, n.e, k18l * n.s));
+    return;
+  }
+  // liquid (rho within 0.1 % of rho_l): the working precision resolves u and p
+  const float tx = (z[5] - z[7]) - (z[6] - z[8]), ty = (z[5] - z[7]) + (z[6] - z[8]);
+  m.rho = K.rho_g + m.phi * K.drl;
+  const float inv = rcp(m.rho);
+  m.jx = ((z[1] - z[3]) + tx) + m.Hx;
+  m.jy = ((z[2] - z[4]) + ty) + m.Hy;
+  m.hx = m.jx * inv;
+  m.hy = m.jy * inv;
+  m.ru = m.jx * m.hx + m.jy * m.hy;
+  m.U = m.hx * Gx + m.hy * Gy;
+  const float znz = ((z[1] + z[3]) + (z[2] + z[4])) + ((z[5] + z[7]) + (z[6] + z[8]));
+  m.Pp = 1.8f * ((znz + m.U) - (float)(2.0 / 3.0) * m.ru);
+}
+
+// Gradient and Laplacian of phi from the shared tile (t: the node's entry, ld: row
+// stride), then the half force, tau, rho, u and p.
+template <typename R>
+__device__ __forceinline__ void mp_macro(const MpParams &P, const R *t, int ld, const R z[9], R fext_x, R fext_y,
+                                         MpMacro<R> &m) {
+  const MpConst<R> &K = KM<R>(P);
+  const R pc = t[0];
+  const R pE = t[1], pW = t[-1], pN = t[ld], pS = t[-ld];
+  const R pNE = t[ld + 1], pNW = t[ld - 1], pSW = t[-ld - 1], pSE = t[-ld + 1];
+  m.phi = pc;
+  // Eq. gradient: sum_i w_i c_i phi_i / (c_s^2 dt) = (3/dx) sum_i w_i e_i phi_i, here 36 sum
+  const R da = pNE - pSW, db = pNW - pSE;
+  m.rx = (R)4 * (pE - pW) + (da - db);
+  m.ry = (R)4 * (pN - pS) + (da + db);
+  // Eq. laplacian: (6/dx^2) sum_i w_i (phi_i - phi), here 36 sum
+  const R l36 = (R)4 * ((pE + pW) + (pN + pS) - (R)4 * pc) + ((pNE + pSW) + (pNW + pSE) - (R)4 * pc);
+  // dt / (2 c) F of Eq. chemical_potential: F = mu grad phi + F_b
+  const R hmu = K.kb * pc * ((pc - (R)1) * (pc - (R)0.5)) - K.kl * l36;
+  m.Hx = hmu * m.rx;
+  m.Hy = hmu * m.ry;
+  if (P.forced) {
+    m.Hx += K.hdt_ic * (K.Fx + fext_x);
+    m.Hy += K.hdt_ic * (K.Fy + fext_y);
+  }
+  // 1 / (36 / (3 / dx) |grad phi|), 0 where the gradient vanishes
+  m.rn = inv_norm(m.rx * m.rx + m.ry * m.ry);
+  recover(P, z, m, K.kg * m.rx, K.kg * m.ry);
+  // tau / dt = nu / (c_s^2 dt) + 1/2 (Eq. eq_kinematic_viscosity)
+  const R tau = P.nu_rule == 0 ? K.tau0 + pc * K.dtau : (K.zg + pc * K.dzeta) * rcp(m.rho) + (R)0.5;
+  m.snu = rcp(tau);
 }
 
 template <typename R>
 __device__ __forceinline__ void collide_h(const MpParams &P, const MpMacro<R> &m, R dpux, R dpuy, R h[5]) {
   const MpConst<R> &K = KM<R>(P);
-  const R c = K.c, inv_cs2 = K.inv_cs2;
-  const R om = K.om_h;
-  const R sfac = K.sfac_h;
-  const R a_int = K.aint_coef * m.phi * ((R)1 - m.phi);  // c_s^2 4 phi (1 - phi) / W
-  const R ax = dpux + a_int * m.nxv, ay = dpuy + a_int * m.nyv;
-  const R phi = m.phi, ux = m.ux, uy = m.uy;
-  R heq_sum = 0;
-#pragma unroll
-  for (int q = 1; q < 5; q++) {
-    const R cxq = c * (R)cx5(q), cyq = c * (R)cy5(q);
-    const R heq = phi * w5<R>(q) * ((R)1 + (cxq * ux + cyq * uy) * inv_cs2);  // Eq. heq_liang
-    const R Sh = w5<R>(q) * (cxq * ax + cyq * ay) * inv_cs2;                    // Eq. source_term_interface
-    heq_sum += heq;
-    h[q] = h[q] - om * (h[q] - heq) + sfac * Sh;
-  }
-  // h_0^eq = phi w_0 = phi - sum_{q>=1} h_q^eq: sum h_eq = phi exactly in the working
-  // precision (in FP32 the rounded weights sum to 1 + 3e-8, a systematic phase gain)
-  h[0] = h[0] - om * (h[0] - (phi - heq_sum));
+  const R d13 = h[1] - h[3], d24 = h[2] - h[4], a13 = h[1] + h[3], a24 = h[2] + h[4];
+  // pairs (Eqs. heq_liang, source_term_interface): even ones relax to phi / 6, odd ones to
+  // phi h / 2, with the source of d_t(phi u) and of the interface flux
+  // (c_s^2 4 phi (1 - phi) / W) n
+  const R p6 = m.phi * ((R)1 / (R)6), flux = K.s2 * (m.phi * ((R)1 - m.phi)) * m.rn;
+  const R px = K.om_h * (p6 - (R)0.5 * a13), py = K.om_h * (p6 - (R)0.5 * a24);
+  const R ox = K.hom_h * (m.phi * m.hx - d13) + K.s1 * dpux + flux * m.rx;
+  const R oy = K.hom_h * (m.phi * m.hy - d24) + K.s1 * dpuy + flux * m.ry;
+  // the rest population takes the remainder: sum h stays phi in the working precision
+  h[0] -= (R)2 * (px + py);
+  h[1] += px + ox;
+  h[3] += px - ox;
+  h[2] += py + oy;
+  h[4] += py - oy;
 }
 
 template <typename R>
 __device__ __forceinline__ void collide_z(const MpParams &P, const MpMacro<R> &m, R z[9]) {
   const MpConst<R> &K = KM<R>(P);
-  const R c = K.c;
-  const R rho = m.rho, ux = m.ux, uy = m.uy;
-  const R Fx = m.Fx, Fy = m.Fy, gx = m.drx, gy = m.dry;
+  // u . grad rho terms: rho_grad holds dt c grad rho
+  const R gx = (R)2 * K.kg * m.rx, gy = (R)2 * K.kg * m.ry;
   if (!P.z_mrt) {
-    // BGK, Eq. eq_lattice_boltzmann_pressure
-    const R inv_cs2 = K.inv_cs2;
-    const R om = m.wb, sfac = ((R)1 - (R)0.5 * m.wb) * K.dt;
-    const R Pp = m.p * K.inv_cs2;
-    const R hu = (R)0.5 * (ux * ux + uy * uy) * inv_cs2;
+    // BGK, Eq. eq_lattice_boltzmann_pressure (lattice-scaled)
+    const R om = m.snu, sfac = (R)1 - (R)0.5 * m.snu;
+    const R hu = (R)1.5 * m.ru;
 #pragma unroll
     for (int q = 0; q < 9; q++) {
-      const R cxq = c * (R)cx9(q), cyq = c * (R)cy9(q);
-      const R cu = cxq * ux + cyq * uy;
-      const R si = w9<R>(q) * (cu * inv_cs2 * ((R)1 + (R)0.5 * cu * inv_cs2) - hu);
-      const R zeq = Pp * (w9<R>(q) - (q == 0 ? (R)1 : (R)0)) + rho * si;  // Eq. zeq_liang
-      const R Fz = w9<R>(q) * ((cxq * Fx + cyq * Fy) + cu * (cxq * gx + cyq * gy)) * inv_cs2;
+      const R ch = (R)cx9(q) * m.hx + (R)cy9(q) * m.hy, cj = (R)cx9(q) * m.jx + (R)cy9(q) * m.jy;
+      const R si = w9<R>(q) * (cj * ((R)3 + (R)4.5 * ch) - hu);                 // rho s_i(u)
+      const R zeq = m.Pp * (w9<R>(q) - (q == 0 ? (R)1 : (R)0)) + si;            // Eq. zeq_liang
+      const R Fz = w9<R>(q) * ((R)6 * ((R)cx9(q) * m.Hx + (R)cy9(q) * m.Hy) +
+                               (R)3 * ch * ((R)cx9(q) * gx + (R)cy9(q) * gy));  // dt F^z_i
       z[q] = z[q] - om * (z[q] - zeq) + sfac * Fz;
     }
     return;
   }
-  // MRT on lattice-scaled moments (see step_sp.cu): equilibrium moments of z_eq
-  // are M f_eq(rho, u) - rho M w + (p/c_s^2)(M w - M e_0); forcing moments of
-  // F_hat^z = w_i [c_i.F + (c_i.u)(c_i.grad rho)] / c_s^2.
-  const R ic = K.ic;
-  const R hx = ux * ic, hy = uy * ic, usq = hx * hx + hy * hy;
-  const R Pp = m.p * K.inv_cs2;
-  const R s14 = (z[1] + z[2]) + (z[3] + z[4]);
-  const R s58 = (z[5] + z[6]) + (z[7] + z[8]);
-  const R m0 = z[0] + s14 + s58;
-  const R m_e = -(R)4 * z[0] - s14 + (R)2 * s58;
-  const R m_ep = (R)4 * z[0] - (R)2 * s14 + s58;
-  const R d58 = z[5] - z[7], d68 = z[6] - z[8];
-  const R m_jx = (z[1] - z[3]) + d58 - d68;
-  const R m_jy = (z[2] - z[4]) + d58 + d68;
-  const R m_qx = (R)2 * (z[3] - z[1]) + d58 - d68;
-  const R m_qy = (R)2 * (z[4] - z[2]) + d58 + d68;
-  const R m_xx = (z[1] + z[3]) - (z[2] + z[4]);
-  const R m_xy = (z[5] + z[7]) - (z[6] + z[8]);
-  const R eq_e = (R)3 * rho * usq + (R)2 * Pp;
-  const R eq_ep = -(R)3 * rho * usq - (R)3 * Pp;
-  const R eq_jx = rho * hx, eq_jy = rho * hy;
-  const R eq_xx = rho * (hx * hx - hy * hy), eq_xy = rho * hx * hy;
-  const R ug = ux * gx + uy * gy;
-  const R F0 = ug, Fep = -ug;
-  const R Fjx = Fx * ic, Fjy = Fy * ic;
-  const R Fxx = (R)(2.0 / 3.0) * (ux * gx - uy * gy), Fxy = (R)(1.0 / 3.0) * (ux * gy + uy * gx);
-  // multiphase [Lambda]_dim (Sec. 3): 1/dt everywhere except omega_q2 (q_x, and
-  // q_y by the isotropic reading) and 1/tau for the stress moments
-  // omega_q2 dt = 3 (2 - omega_nu dt) / (3 - omega_nu dt), omega_nu dt = dt / tau (Sec. 3)
-  const R snu = m.wb;
-  const R sq = qdiv((R)3 * ((R)2 - snu), (R)3 - snu);
+  // MRT, multiphase [Lambda]_dim (Sec. 3): rate 1/dt everywhere except omega_q2 (q_x, and
+  // q_y by the isotropic reading) and 1/tau for the stress moments; omega_q2 dt = 3 (2 -
+  // omega_nu dt) / (3 - omega_nu dt).  At rate 1 a moment goes to its equilibrium plus half
+  // its forcing: sum z' = U, e' = 3 ru + 2 Pp, eps' = -3 ru - 3 Pp - U, j' = j + H.  So the
+  // even pairs keep only the stress of z and the odd ones only q.
+  const R d13 = z[1] - z[3], d24 = z[2] - z[4], d57 = z[5] - z[7], d68 = z[6] - z[8];
+  const R xx = (z[1] + z[3]) - (z[2] + z[4]), xy = (z[5] + z[7]) - (z[6] + z[8]);
+  const R snu = m.snu, sq = ((R)6 - (R)3 * snu) * rcp((R)3 - snu);
   const R sqy = P.qy_literal ? (R)1 : sq;
-  const R rdt = K.dt, one = (R)1, half = (R)0.5;
-  const R d0 = m0 - half * rdt * F0;                 // s = 1: (m - 0) - (1 - 1/2) dt F
-  const R d_e = (m_e - eq_e);                        // F_e = 0
-  const R d_ep = (m_ep - eq_ep) - half * rdt * Fep;
-  const R d_jx = (m_jx - eq_jx) - half * rdt * Fjx;
-  const R d_jy = (m_jy - eq_jy) - half * rdt * Fjy;
-  const R d_qx = sq * (m_qx + eq_jx) + (one - half * sq) * rdt * Fjx;   // eq_qx = -rho u_x/c, F_qx = -F_x/c
-  const R d_qy = sqy * (m_qy + eq_jy) + (one - half * sqy) * rdt * Fjy;
-  const R d_xx = snu * (m_xx - eq_xx) - (one - half * snu) * rdt * Fxx;
-  const R d_xy = snu * (m_xy - eq_xy) - (one - half * snu) * rdt * Fxy;
-  const R a0 = d0 * ((R)1 / (R)9);
-  const R a1 = d_e * ((R)1 / (R)36), a2 = d_ep * ((R)1 / (R)36);
-  const R a3 = d_jx * ((R)1 / (R)6), a4 = d_qx * ((R)1 / (R)12);
-  const R a5 = d_jy * ((R)1 / (R)6), a6 = d_qy * ((R)1 / (R)12);
-  const R a7 = d_xx * (R)0.25, a8 = d_xy * (R)0.25;
-  const R ax = a0 - a1 - (R)2 * a2;
-  const R dg = a0 + (R)2 * a1 + a2;
-  z[0] -= a0 + (R)4 * (a2 - a1);
-  z[1] -= ax + a3 - (R)2 * a4 + a7;
-  z[2] -= ax + a5 - (R)2 * a6 - a7;
-  z[3] -= ax - a3 + (R)2 * a4 + a7;
-  z[4] -= ax - a5 + (R)2 * a6 - a7;
-  const R p34 = a3 + a4, p56 = a5 + a6;
-  z[5] -= dg + p34 + p56 + a8;
-  z[6] -= dg - p34 + p56 - a8;
-  z[7] -= dg - p34 - p56 + a8;
-  z[8] -= dg + p34 - p56 - a8;
+  const R r3 = m.ru * ((R)1 / (R)12), p36 = m.Pp * ((R)1 / (R)36), u12 = m.U * ((R)1 / (R)12);
+  const R e4 = (R)2 * u12 + (r3 + (R)4 * p36), e8 = u12 + (r3 + p36);
+  const R xx0 = m.jx * m.hx, rxx = xx0 - m.jy * m.hy, rxy = m.jx * m.hy;
+  const R f3 = ((R)1 - (R)0.5 * snu) * ((R)1 / (R)3);
+  const R gxx = m.hx * gx, Fxx = (R)2 * (gxx - m.hy * gy), Fxy = m.hx * gy + m.hy * gx;
+  const R X = (R)0.25 * (xx + snu * (rxx - xx) + f3 * Fxx), Y = (R)0.25 * (xy + snu * (rxy - xy) + f3 * Fxy);
+  const R qx = ((d57 - d68) - (R)2 * d13), qy = ((d57 + d68) - (R)2 * d24);
+  const R jx = m.jx + m.Hx, jy = m.jy + m.Hy;
+  const R qxn = qx - (sq * (qx + m.jx) + ((R)2 - sq) * m.Hx), qyn = qy - (sqy * (qy + m.jy) + ((R)2 - sqy) * m.Hy);
+  const R Qx = (jx - qxn) * ((R)1 / (R)6), Qy = (jy - qyn) * ((R)1 / (R)6);
+  const R bx = (R)0.5 * jx - Qx, by = (R)0.5 * jy - Qy;
+  const R w = (R)0.5 * (bx + by), v = (R)0.5 * (by - bx);
+  const R P13 = e4 + X, P24 = e4 - X, P57 = e8 + Y, P68 = e8 - Y;
+  z[0] = m.U - (R)4 * (e4 + e8);
+  z[1] = P13 + Qx;
+  z[3] = P13 - Qx;
+  z[2] = P24 + Qy;
+  z[4] = P24 - Qy;
+  z[5] = P57 + w;
+  z[7] = P57 - w;
+  z[6] = P68 + v;
+  z[8] = P68 - v;
 }
 
 enum { MODE_STEP = 0, MODE_MOMENTS = 2, MODE_INTEGRALS = 3 };
 
-template <int BY>
 __device__ __forceinline__ void reduce4_block(double v[4], double *out) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -298,12 +349,12 @@ __device__ __forceinline__ void reduce4_block(double v[4], double *out) {
     v[3] += __shfl_down_sync(0xffffffffu, v[3], o);
   }
   __shared__ double sh[8][4];
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x, nw = (blockDim.x * blockDim.y) / 32;
   if ((tid & 31) == 0) { sh[tid >> 5][0] = v[0]; sh[tid >> 5][1] = v[1]; sh[tid >> 5][2] = v[2]; sh[tid >> 5][3] = v[3]; }
   __syncthreads();
   if (tid == 0) {
     double a = 0, b = 0, mx = 0, cnt = 0;
-    for (int w = 0; w < (BX * BY) / 32; w++) { a += sh[w][0]; b += sh[w][1]; mx = fmax(mx, sh[w][2]); cnt += sh[w][3]; }
+    for (int w = 0; w < nw; w++) { a += sh[w][0]; b += sh[w][1]; mx = fmax(mx, sh[w][2]); cnt += sh[w][3]; }
     out[0] = a; out[1] = b; out[2] = mx; out[3] = cnt;
   }
 }
@@ -315,36 +366,25 @@ __device__ __forceinline__ void reduce4_block(double v[4], double *out) {
 #define LBM_MP_FP32_BLOCKS_PER_SM 5
 #endif
 
-// pass 2 (and its init / moments / integrals variants)
+template <int BY> constexpr int mp_threads() { return BY ? BX * BY : 32; }
+
+// One step (and its moments / integrals variants).  BY = 0: one-warp blocks of whole rows
+// (narrow grids).
 template <int PREC, int MODE, int BY>
-__global__ void __launch_bounds__(BX * BY, (PREC == 1 && BY == 8) ? LBM_MP_FP32_BLOCKS_PER_SM : 0) k_mp_collide(const MpParams P, const double *A, const double *UX,
-                                                         const double *UY, const double *B, unsigned mask,
-                                                         double *out) {
+__global__ void __launch_bounds__(mp_threads<BY>(), (PREC == 1 && BY == 8) ? LBM_MP_FP32_BLOCKS_PER_SM : 0)
+k_mp_collide(const MpParams P, unsigned mask, double *out) {
   typedef typename Prec<PREC>::S S;
   typedef typename Prec<PREC>::R R;
-  __shared__ R tile[BY + 2][BX + 2];
-  const int i0 = blockIdx.x * BX, j0 = blockIdx.y * BY;
-  const int tid = threadIdx.y * BX + threadIdx.x;
-  const int i = i0 + threadIdx.x, j = j0 + threadIdx.y;
-  const bool live = (i < P.nx) && (j < P.ny);
+  __shared__ R tile[BY ? (BY + 2) * (BX + 2) : kNarrowTile];
   const S *src = (const S *)P.src;
-  // phi = sum_i h_i (Eq. zero_moment_h) of the tile and of a one-node periodic halo,
-  // from pulled h: this node's h stays in registers for its collision
-  // a block whose tile, halo and their pull sources stay off the periodic seams
-  // (the bulk of the grid) pulls with plain offsets: no wrap, no modulo
-  const bool inner = !P.local && i0 >= 2 && j0 >= 2 && i0 + BX + 2 <= P.nx && j0 + BY + 2 <= P.ny;
-  R h[5];
-  if (inner) {
-    pull_h_at<S, R>(P, src + ((long long)j * P.pitch + i), h);
-  } else {
-    pull_h<S, R>(P, src, stencil_node(i, P.nx, P.xwall), stencil_node(j, P.ny, P.ywall), h);
-  }
-  // the node's z, (phi u)_prev and force do not depend on the tile: their loads are
-  // issued here, so that they are in flight during the halo pulls and the barrier
-  const long long n = (long long)j * P.pitch + i;
-  R z[9];
+  int i, j, ld, at;  // node, row stride of the tile, the node's entry in it
+  bool live, inner = false;
+  // phi = sum_i h_i (Eq. zero_moment_h) of the tile and of a one-node halo, from pulled h:
+  // this node's h stays in registers for its collision.  The node's z, (phi u)_prev and
+  // force do not depend on the tile: their loads are issued before the barrier
+  R h[5], z[9];
   R prevx = 0, prevy = 0, fex = 0, fey = 0;
-  if (live) {
+  auto load_node = [&](long long n) {
     if (P.force) {
       fex = (R)((const S *)P.force)[n];
       fey = (R)((const S *)P.force)[P.plane + n];
@@ -355,32 +395,73 @@ __global__ void __launch_bounds__(BX * BY, (PREC == 1 && BY == 8) ? LBM_MP_FP32_
       prevx = (R)src[14ll * P.plane + n];
       prevy = (R)src[15ll * P.plane + n];
     }
-  }
-  tile[threadIdx.y + 1][threadIdx.x + 1] = (h[0] + h[1]) + (h[2] + h[3]) + h[4];
-  constexpr int kHalo = 2 * (BX + 2) + 2 * BY;
-  for (int t = tid; t < kHalo; t += BX * BY) {
-    int tx, ty;
-    if (t < BX + 2) { tx = t; ty = 0; }                            // row below the tile
-    else if (t < 2 * (BX + 2)) { tx = t - (BX + 2); ty = BY + 1; }  // row above
-    else if (t < 2 * (BX + 2) + BY) { tx = 0; ty = t - 2 * (BX + 2) + 1; }  // left column
-    else { tx = BX + 1; ty = t - 2 * (BX + 2) - BY + 1; }           // right column
-    R hh[5];
-    if (inner) {
-      pull_h_at<S, R>(P, src + ((long long)(j0 + ty - 1) * P.pitch + (i0 + tx - 1)), hh);
-    } else {
-      pull_h<S, R>(P, src, stencil_node(i0 + tx - 1, P.nx, P.xwall), stencil_node(j0 + ty - 1, P.ny, P.ywall), hh);
+  };
+  auto sum5 = [](const R *a) { return (a[0] + a[1]) + (a[2] + a[3]) + a[4]; };
+  if (BY == 0) {
+    const int nx = P.nx, rows = 32 / nx, j0 = blockIdx.x * rows, r = min(rows, P.ny - j0);
+    const int ty = threadIdx.x / nx;
+    ld = nx + 2;
+    i = threadIdx.x - ty * nx;
+    j = j0 + ty;
+    at = (ty + 1) * ld + i + 1;
+    live = ty < r;
+    // an entry and, for the first and last column, its image beside the row
+    auto put = [&](int row, int col, R phi) {
+      tile[row * ld + col + 1] = phi;
+      if (col == 0) tile[row * ld + (P.xwall ? 0 : nx + 1)] = phi;
+      if (col == nx - 1) tile[row * ld + (P.xwall ? nx + 1 : 0)] = phi;
+    };
+    if (live) {
+      pull_h<S, R>(P, src, i, j, h);
+      load_node((long long)j * P.pitch + i);
+      put(ty + 1, i, sum5(h));
     }
-    tile[ty][tx] = (hh[0] + hh[1]) + (hh[2] + hh[3]) + hh[4];
+    for (int t = threadIdx.x; t < 2 * nx; t += 32) {  // the rows below and above the block
+      const int up = t >= nx, col = up ? t - nx : t;
+      R hh[5];
+      pull_h<S, R>(P, src, col, stencil_node(up ? j0 + r : j0 - 1, P.ny, P.ywall), hh);
+      put(up ? r + 1 : 0, col, sum5(hh));
+    }
+  } else {
+    const int i0 = blockIdx.x * BX, j0 = blockIdx.y * BY;
+    const int tid = threadIdx.y * BX + threadIdx.x;
+    i = i0 + threadIdx.x;
+    j = j0 + threadIdx.y;
+    ld = BX + 2;
+    at = (threadIdx.y + 1) * (BX + 2) + threadIdx.x + 1;
+    live = (i < P.nx) && (j < P.ny);
+    // a block whose tile, halo and their pull sources stay off the periodic seams
+    // (the bulk of the grid) pulls with plain offsets: no wrap, no modulo
+    inner = !P.local && i0 >= 2 && j0 >= 2 && i0 + BX + 2 <= P.nx && j0 + BY + 2 <= P.ny;
+    if (inner) pull_h_at<S, R>(P, src + ((long long)j * P.pitch + i), h);
+    else pull_h<S, R>(P, src, stencil_node(i, P.nx, P.xwall), stencil_node(j, P.ny, P.ywall), h);
+    if (live) load_node((long long)j * P.pitch + i);
+    tile[at] = sum5(h);
+    constexpr int kHalo = 2 * (BX + 2) + 2 * BY;
+    for (int t = tid; t < kHalo; t += BX * BY) {
+      int tx, ty;
+      if (t < BX + 2) { tx = t; ty = 0; }                            // row below the tile
+      else if (t < 2 * (BX + 2)) { tx = t - (BX + 2); ty = BY + 1; }  // row above
+      else if (t < 2 * (BX + 2) + BY) { tx = 0; ty = t - 2 * (BX + 2) + 1; }  // left column
+      else { tx = BX + 1; ty = t - 2 * (BX + 2) - BY + 1; }           // right column
+      R hh[5];
+      if (inner) {
+        pull_h_at<S, R>(P, src + ((long long)(j0 + ty - 1) * P.pitch + (i0 + tx - 1)), hh);
+      } else {
+        pull_h<S, R>(P, src, stencil_node(i0 + tx - 1, P.nx, P.xwall), stencil_node(j0 + ty - 1, P.ny, P.ywall), hh);
+      }
+      tile[ty * (BX + 2) + tx] = sum5(hh);
+    }
   }
   __syncthreads();
   double red[4] = {0.0, 0.0, 0.0, 0.0};
   if (live) {
+    const long long n = (long long)j * P.pitch + i;
     MpMacro<R> m;
-    mp_macro<R>(P, tile, threadIdx.x + 1, threadIdx.y + 1, z, fex, fey, m);
+    mp_macro<R>(P, tile + at, BY ? BX + 2 : ld, z, fex, fey, m);
     if (MODE == MODE_STEP) {
-      const R pux = m.phi * m.ux, puy = m.phi * m.uy;
-      const R dpux = (pux - prevx) * KM<R>(P).inv_dt, dpuy = (puy - prevy) * KM<R>(P).inv_dt;  // explicit Euler d_t(phi u)
-      collide_h<R>(P, m, dpux, dpuy, h);
+      const R pux = m.phi * (KM<R>(P).c * m.hx), puy = m.phi * (KM<R>(P).c * m.hy);
+      collide_h<R>(P, m, pux - prevx, puy - prevy, h);  // explicit Euler d_t(phi u)
       collide_z<R>(P, m, z);
       S *dst = (S *)P.dst;
 #pragma unroll
@@ -393,15 +474,15 @@ __global__ void __launch_bounds__(BX * BY, (PREC == 1 && BY == 8) ? LBM_MP_FP32_
       const long long N = (long long)P.nx * P.ny, k = (long long)j * P.nx + i;
       int slot = 0;
       if (mask & 1u) out[(slot++) * N + k] = (double)m.rho;
-      if (mask & 2u) out[(slot++) * N + k] = (double)m.ux;
-      if (mask & 4u) out[(slot++) * N + k] = (double)m.uy;
+      if (mask & 2u) out[(slot++) * N + k] = P.c * (double)m.hx;
+      if (mask & 4u) out[(slot++) * N + k] = P.c * (double)m.hy;
       if (mask & 8u) out[(slot++) * N + k] = 0.0;
-      if (mask & 16u) out[(slot++) * N + k] = (double)m.p;
+      if (mask & 16u) out[(slot++) * N + k] = P.cs2 * (double)m.Pp;
       if (mask & 32u) out[(slot++) * N + k] = (double)m.phi;
     } else {
-      const double ux = (double)m.ux, uy = (double)m.uy, rho = (double)m.rho, p = (double)m.p;
+      const double ux = P.c * (double)m.hx, uy = P.c * (double)m.hy, rho = (double)m.rho, pr = (double)m.Pp;
       const double umag = sqrt(ux * ux + uy * uy);
-      const bool bad = !isfinite(rho) || !isfinite(umag) || !isfinite(p) || umag >= P.c;
+      const bool bad = !isfinite(rho) || !isfinite(umag) || !isfinite(pr) || umag >= P.c;
       // a bad node (non-finite, or |u| >= c) is counted and adds nothing else
       red[0] = bad ? 0.0 : rho * P.dx * P.dx;
       red[1] = bad ? 0.0 : (double)m.phi;
@@ -409,7 +490,7 @@ __global__ void __launch_bounds__(BX * BY, (PREC == 1 && BY == 8) ? LBM_MP_FP32_
       red[3] = bad ? 1.0 : 0.0;
     }
   }
-  if (MODE == MODE_INTEGRALS) reduce4_block<BY>(red, out + 4ll * (blockIdx.y * gridDim.x + blockIdx.x));
+  if (MODE == MODE_INTEGRALS) reduce4_block(red, out + 4ll * (blockIdx.y * gridDim.x + blockIdx.x));
 }
 
 __global__ void k_mp_final(const double *partials, int nb, double *out4) {
@@ -458,15 +539,23 @@ __global__ void k_mp_init(const MpParams P, const double *A, const double *UX, c
   dst[15ll * P.plane + n] = (S)(ph * v0);
 }
 
-dim3 mp_grid(int nx, int ny, int by) { return dim3((nx + BX - 1) / BX, (ny + by - 1) / by); }
-int mp_rows(int nx, int ny) { return (int)(mp_grid(nx, ny, 8).x * mp_grid(nx, ny, 8).y) >= kSmallGridBlocks ? 8 : 2; }
+// Blocks of a launch: rows BY of a tile by size, 0 (whole rows) on narrow grids.
+dim3 mp_grid(int nx, int ny, int by) {
+  if (by == 0) return dim3((ny + 32 / nx - 1) / (32 / nx));
+  return dim3((nx + BX - 1) / BX, (ny + by - 1) / by);
+}
+int mp_rows(int nx, int ny) {
+  if (nx <= kNarrow) return 0;
+  return (int)(mp_grid(nx, ny, 8).x * mp_grid(nx, ny, 8).y) >= kSmallGridBlocks ? 8 : 2;
+}
 
 template <int PREC, int MODE>
 void launch_collide(const MpParams &P, unsigned mask, double *out, cudaStream_t s) {
   const int by = mp_rows(P.nx, P.ny);
   const dim3 g = mp_grid(P.nx, P.ny, by);
-  if (by == 8) k_mp_collide<PREC, MODE, 8><<<g, dim3(BX, 8), 0, s>>>(P, nullptr, nullptr, nullptr, nullptr, mask, out);
-  else k_mp_collide<PREC, MODE, 2><<<g, dim3(BX, 2), 0, s>>>(P, nullptr, nullptr, nullptr, nullptr, mask, out);
+  if (by == 8) k_mp_collide<PREC, MODE, 8><<<g, dim3(BX, 8), 0, s>>>(P, mask, out);
+  else if (by == 2) k_mp_collide<PREC, MODE, 2><<<g, dim3(BX, 2), 0, s>>>(P, mask, out);
+  else k_mp_collide<PREC, MODE, 0><<<g, 32, 0, s>>>(P, mask, out);
 }
 
 }  // namespace
