@@ -33,55 +33,85 @@ namespace {
 
 __device__ __forceinline__ long long nidx(const SpParams &P, int i, int j) { return (long long)j * P.pitch + i; }
 
-// The link arriving at node (i, j) along q is an ordinary streaming link (its
-// source is inside the domain or wraps periodically).
-__device__ __forceinline__ bool streams_in(const SpParams &P, int i, int j, int cx, int cy, int xper, int yper) {
-  return entry_side(i, j, cx, cy, P.nx, P.ny, xper, yper) < 0;
-}
-
-// d(pre_p)/d(u_w) of the anti-BB outlet rule for outgoing direction o.
-template <typename R>
-__device__ __forceinline__ void dpre_duw(const SpParams &P, int o, R rw, R uwx, R uwy, R &gx, R &gy) {
-  const R c = K<R>(P).c, ics2 = K<R>(P).inv_cs2;
-  const R cx = c * (R)cx9(o), cy = c * (R)cy9(o);
-  const R cu = cx * uwx + cy * uwy;
-  const R k = (R)2 * w9<R>(o) * rw;
-  gx = k * (cu * cx * ics2 * ics2 - uwx * ics2);
-  gy = k * (cu * cy * ics2 * ics2 - uwy * ics2);
-}
-
-// G = sum over the outlet's unknown populations p of Lam_pre_p * d(pre_p)/d(u_w) at
-// boundary node (bi, bj) of pressure side s; also returns u_w inputs.
+// The outlet's velocity extrapolation u_w = 1.5 u(x_b) - 0.5 u(x_b-1) seen from the node
+// (i, j) itself (`on`, the boundary node of side s) or from its inner neighbour: the
+// adjoint of u_w, G = sum over the side's unknown populations p of Lam_pre_p
+// d(pre_p)/d(u_w), times d(u_w)/d(u at this node) / rho; and this node's velocity.
 template <typename S, typename R>
-__device__ void outlet_G(const SpParams &P, const S *Xt, const R *LPn, int s, int bi, int bj, R &Gx, R &Gy) {
-  const int ii = bi + (s == 0) - (s == 1), jj = bj + (s == 2) - (s == 3);
-  R ub, vb, ui, vi;
-  post_velocity<S, R>(P, Xt, bi, bj, ub, vb);
-  post_velocity<S, R>(P, Xt, ii, jj, ui, vi);
-  const R uwx = ub + (R)0.5 * (ub - ui), uwy = vb + (R)0.5 * (vb - vi);
+__device__ __forceinline__ void outlet_adjoint(const SpParams &P, const S *Xt, const R *LPn, int s, bool on, int i, int j,
+                                               R &Gx, R &Gy, R &ux, R &uy) {
+  const int di = (s == 0) - (s == 1), dj = (s == 2) - (s == 3);  // inward
+  const int bi = on ? i : i - di, bj = on ? j : j - dj;
+  R ub, vb, ui, vi, rb, ri;
+  post_velocity<S, R>(P, Xt, bi, bj, ub, vb, rb);
+  post_velocity<S, R>(P, Xt, bi + di, bj + dj, ui, vi, ri);
+  const R wx = ub + (R)0.5 * (ub - ui), wy = vb + (R)0.5 * (vb - vi);
+  const R c = K<R>(P).c, ics2 = K<R>(P).inv_cs2, rw = K<R>(P).rho_w[s];
+  const long long nb = nidx(P, bi, bj);
   Gx = 0;
   Gy = 0;
-  const long long nb = nidx(P, bi, bj);
 #pragma unroll
-  for (int p = 0; p < 9; p++) {
+  for (int p = 1; p < 9; p++) {
     if (entry_side(bi, bj, cx9(p), cy9(p), P.nx, P.ny, P.xper, P.yper) != s) continue;
-    R gx, gy;
-    dpre_duw<R>(P, opp9(p), K<R>(P).rho_w[s], uwx, uwy, gx, gy);
-    const R lam = LPn[p * P.plane + nb];
-    Gx += lam * gx;
-    Gy += lam * gy;
+    // d/d u_w of the anti-BB rule 2 w rho_w ((c.u)^2 / 2 c_s^4 - u^2 / 2 c_s^2)
+    const R cx = c * (R)cx9(p), cy = c * (R)cy9(p);
+    const R k = (R)2 * w9<R>(p) * rw * ics2 * LPn[p * P.plane + nb], cu = (cx * wx + cy * wy) * ics2;
+    Gx += k * (cu * cx - wx);
+    Gy += k * (cu * cy - wy);
   }
+  const R coef = (on ? (R)1.5 : (R)-0.5) / (on ? rb : ri);
+  Gx *= coef;
+  Gy *= coef;
+  ux = on ? ub : ui;
+  uy = on ? vb : vi;
 }
 
-// Post-collision density and velocity of X at a node (for d u / d X).
+// Lam_X(t) = P^T Lam_pre(t+1) at a node within two cells of a side.  Population q of this
+// node is consumed by the streaming neighbour along c_q, or where that link leaves the
+// domain by the node's own reflected link opp(q) of that side; the outlet and the thermal
+// outflow add theirs.
 template <typename S, typename R>
-__device__ __forceinline__ void post_rho_u(const SpParams &P, const S *X, int i, int j, R &rho, R &ux, R &uy) {
+__device__ __forceinline__ void gather_frame(const SpParams &P, const S *Xt, const R *LPn, int i, int j, R lx[9], R lg[5],
+                                             double *grad_flux2, double *grad_flux3) {
   const long long n = nidx(P, i, j);
-  R s = 0;
+  const NodeSides b = node_sides(P, i, j, P.xper, P.yper);
 #pragma unroll
-  for (int q = 0; q < 9; q++) s += (R)X[q * P.plane + n];
-  rho = K<R>(P).rho0 + s;
-  post_velocity<S, R>(P, X, i, j, ux, uy);
+  for (int q = 0; q < 9; q++) {
+    const int p = opp9(q), cx = cx9(p), cy = cy9(p);
+    const bool by_x = enters<false>(b, side_x(cx), cx, cy, 0), by_y = enters<false>(b, side_y(cy), cx, cy, 0);
+    const int kind = by_y ? P.side[side_y(cy)].kind : P.side[side_x(cx)].kind;
+    // (the streaming source of opp(q) is the consumer of q)
+    const R v = LPn[by_x || by_y ? p * P.plane + n : q * P.plane + stream_at(b, i, cx, cy)];
+    lx[q] = (by_x || by_y) && kind == BC_PRESSURE ? -v : v;
+  }
+#pragma unroll 1
+  for (int s = 0; s < 4; s++) {
+    if (P.side[s].kind != BC_PRESSURE) continue;
+    const int d = s == 0 ? i : s == 1 ? P.nx - 1 - i : s == 2 ? j : P.ny - 1 - j;  // distance from the side
+    if (d > 1) continue;
+    R Gx, Gy, ux, uy;
+    outlet_adjoint<S, R>(P, Xt, LPn, s, d == 0, i, j, Gx, Gy, ux, uy);
+    const R c = K<R>(P).c;
+#pragma unroll
+    for (int q = 0; q < 9; q++) lx[q] += Gx * (c * (R)cx9(q) - ux) + Gy * (c * (R)cy9(q) - uy);
+  }
+  const R *LPng = LPn + (long long)P.gbase * P.plane;
+  const NodeSides t = node_sides(P, i, j, P.txper, P.typer);
+#pragma unroll
+  for (int q = 0; q < 5; q++) {
+    const int p = opp5(q), cx = cx5(p), cy = cy5(p);
+    const int s = cx != 0 ? side_x(cx) : side_y(cy);  // an axis link has one side
+    const bool out = enters<false>(t, s, cx, cy, 0);
+    const int tk = P.side[s].tkind;
+    R v = LPng[out ? p * P.plane + n : q * P.plane + stream_at(t, i, cx, cy)];
+    if (out) v = tk == TBC_FLUX ? v : tk == TBC_TEMP ? -v : (R)0;
+    // wall heat flux gradient: pre_p = X_q + flux_coef q''(a) on flux sides
+    if (out && s >= 2 && tk == TBC_FLUX) (s == 2 ? grad_flux2 : grad_flux3)[i] += P.flux_coef * (double)v;
+    // outflow consumer: the unknown q of an outflow side reads X_q of this node
+    const int sq = cx != 0 ? side_x(-cx) : side_y(-cy);
+    if (enters<false>(t, sq, -cx, -cy, 0) && P.side[sq].tkind == TBC_OUTFLOW) v += LPng[q * P.plane + n];
+    lg[q] = v;
+  }
 }
 
 }  // namespace
@@ -134,227 +164,194 @@ __global__ void k_adj_loss(const SpParams P, const double *Ttarget, R *LP, doubl
   grad_add_fp64<R>(grad_qdot, n, 0.5 * P.dt * dLdT);
 }
 
+// The node's share of a reverse step after Lam_X(t) is known: pre(t) from X_{t-1}, the
+// transposed collisions (the pair forms of sp_device.cuh, reversed line by line), the
+// parameter gradients and Lam_pre(t).  Returns this node's share of dL/dnu (cn, cq: ds_nu
+// / dnu and ds_q / dnu).
+template <typename S, typename R, bool INNER>
+__device__ __forceinline__ R reverse_node(const SpParams &P, int i, int j, R lx[9], R lg[5], R *LP, double *grad_qdot,
+                                          R cn, R cq) {
+  const long long n = nidx(P, i, j);
+  const SpConst<R> &k = K<R>(P);
+  const S *src = (const S *)P.src;
+  R f[9], g[5];
+  if (INNER) {  // P.local (t = 0): the node's own values are the pre-collision state
+    const S *gs = src + (long long)P.gbase * P.plane;
+    const long long row = P.local ? 0 : P.pitch;
+    const int col = P.local ? 0 : 1;
+#pragma unroll
+    for (int q = 0; q < 9; q++) f[q] = (R)src[q * P.plane + n - cy9(q) * row - cx9(q) * col];
+#pragma unroll
+    for (int q = 0; q < 5; q++) g[q] = (R)gs[q * P.plane + n - cy5(q) * row - cx5(q) * col];
+  } else {
+    const bool interior = !P.local && (i > 0) && (i < P.nx - 1) && (j > 0) && (j < P.ny - 1);
+    pull_f<S, R>(P, src, i, j, interior, f);
+    pull_g<S, R>(P, src, i, j, interior, g);
+  }
+  Macro<R> m;
+  load_sources<S, R>(P, n, m);
+  moments<R, FLOW_MRT, TH_MRT>(P, f, g, m);
+  const R inv = recip(m.rho), hx = m.hx, hy = m.hy;
+  const R half = (R)0.5, two = (R)2;
+
+  // thermal D2Q5 MRT: S = sum g + dt qdot to the weights, e = d - T h at rate s_T
+  const R m13 = lg[1] - lg[3], m24 = lg[2] - lg[4];
+  const R X = -k.hsT * m13, Y = -k.hsT * m24;
+  // (2 l0 + l1 + .. + l4) / 6 from the differences, so that equal ones stay exactly equal
+  const R lS = lg[0] + (((lg[1] + lg[3]) + (lg[2] + lg[4])) - (R)4 * lg[0]) * ((R)1 / (R)6);
+  const R lT = -(hx * X + hy * Y);
+  grad_add(grad_qdot, n, (R)(k.dt * lS + k.hdt * lT));
+  R Hx = -m.T * X, Hy = -m.T * Y;  // adjoint of h through the advected heat
+  const R lsum = lS + lT;
+  R *LPg = LP + (long long)P.gbase * P.plane;
+  const R kT = half - k.hsT;
+  LPg[n] = lsum;
+  LPg[1 * P.plane + n] = lsum + kT * m13;
+  LPg[3 * P.plane + n] = lsum - kT * m13;
+  LPg[2 * P.plane + n] = lsum + kT * m24;
+  LPg[4 * P.plane + n] = lsum - kT * m24;
+
+  // momentum D2Q9 MRT: adjoints of the pair changes ...
+  const R p13 = lx[1] + lx[3], o13 = lx[1] - lx[3], p24 = lx[2] + lx[4], o24 = lx[2] - lx[4];
+  const R p57 = lx[5] + lx[7], o57 = lx[5] - lx[7], p68 = lx[6] + lx[8], o68 = lx[6] - lx[8];
+  const R A4 = p13 + p24, AX = p13 - p24, A8 = p57 + p68, AY = p57 - p68;
+  const R Ox = o13 - half * (o57 - o68), Oy = o24 - half * (o57 + o68);
+  const R kx = k.kq * Ox, ky = k.kq * Oy, bX = k.kn * AX, bY = k.kn * AY;
+  // ... of the energies (s4, s8: what is left of half the pair sums; l0: of f_0) ...
+  R s4 = 0, s8 = 0, l0 = 0, lr, lru;
+  if (P.unit_e) {
+    const R E4 = A4 - (R)4 * lx[0], E8 = A8 - (R)4 * lx[0];
+    lr = lx[0] + (E4 * ((R)1 / (R)9) + E8 * ((R)1 / (R)36));
+    lru = (E4 + E8) * ((R)1 / (R)12);
+  } else {
+    const R c1 = k.ke * ((A4 - two * A8) + (R)4 * lx[0]), c2 = k.kep * ((two * A4 - A8) - (R)4 * lx[0]);
+    lr = 0;
+    lru = c2 - (R)3 * c1;
+    l0 = lx[0] + (c2 - two * c1);
+    s4 = (R)0.25 * A4 + (c1 - c2);
+    s8 = (R)0.25 * A8 + (R)4 * c1;
+  }
+  // ... of the stress: rho u^2 terms through j and rho ...
+  const R u2 = two * (lru + bX), v2 = two * (lru - bX);
+  R Jx = u2 * hx + bY * hy, Jy = v2 * hy + bY * hx;
+  lr -= half * (hx * Jx + hy * Jy);
+  // d L / d s_nu and d L / d s_q
+  const R xx = (f[1] + f[3]) - (f[2] + f[4]), xy = (f[5] + f[7]) - (f[6] + f[8]);
+  const R tx = (f[5] - f[7]) - (f[6] - f[8]), ty = (f[5] - f[7]) + (f[6] - f[8]);
+  const R xx0 = m.jx * hx;
+  R dn = AX * ((xx0 - m.jy * hy) - xx) + AY * (m.jx * hy - xy);
+  R dq = Ox * ((tx + m.jx) - two * (f[1] - f[3])) + Oy * ((ty + m.jy) - two * (f[2] - f[4]));
+  if (P.forced) {
+    const R px = m.Fx * k.inv_c, py = m.Fy * k.inv_c;
+    const R gX = k.gn * AX, gY = half * k.gn * AY;
+    R lF = k.g4 * A4 + k.g8 * A8 - (R)4 * (k.g4 + k.g8) * lx[0];
+    Hx += (lF + gX) * px + gY * py;
+    Hy += (lF - gX) * py + gY * px;
+    dn -= k.dt * (AX * (hx * px - hy * py) + half * AY * (hx * py + hy * px));
+    dq -= half * k.dt * (Ox * px + Oy * py);
+  }
+  // ... and of h = j / rho
+  Hx *= inv;
+  Hy *= inv;
+  lr -= hx * Hx + hy * Hy;
+  Jx += kx + Hx;
+  Jy += ky + Hy;
+  const R qx = Jx + kx, qy = Jy + ky;  // of the diagonals' share of the first moment
+  const R d13 = half * o13 + (Jx - two * kx), d24 = half * o24 + (Jy - two * ky);
+  const R d57 = half * o57 + (qy + qx), d68 = half * o68 + (qy - qx);
+  const R kr = (R)0.25 - k.kn;
+  const R e4 = lr + s4, e8 = lr + s8, a13 = e4 + kr * AX, a24 = e4 - kr * AX, a57 = e8 + kr * AY, a68 = e8 - kr * AY;
+  LP[n] = lr + l0;
+  LP[1 * P.plane + n] = a13 + d13;
+  LP[3 * P.plane + n] = a13 - d13;
+  LP[2 * P.plane + n] = a24 + d24;
+  LP[4 * P.plane + n] = a24 - d24;
+  LP[5 * P.plane + n] = a57 + d57;
+  LP[7 * P.plane + n] = a57 - d57;
+  LP[6 * P.plane + n] = a68 + d68;
+  LP[8 * P.plane + n] = a68 - d68;
+  return cn * ((R)0.25 * dn) + cq * (dq * ((R)1 / (R)6));
+}
+
+// Nodes within two cells of a side, each once: the rows j < 2 and j >= ny - 2, then the
+// columns i < 2 and i >= nx - 2 between them.
+__host__ __device__ inline int adj_frame_nodes(int nx, int ny) {
+  const int rows = ny < 4 ? ny : 4, cols = nx < 4 ? nx : 4;
+  return rows * nx + cols * (ny - rows);
+}
+__device__ __forceinline__ bool adj_frame_node(int nx, int ny, int f, int &i, int &j) {
+  const int rows = ny < 4 ? ny : 4, cols = nx < 4 ? nx : 4, inner = ny - rows;
+  if (f < rows * nx) {
+    const int r = f / nx;
+    i = f - r * nx;
+    j = ny < 4 || r < 2 ? r : ny - 4 + r;
+    return true;
+  }
+  f -= rows * nx;
+  if (inner <= 0 || f >= cols * inner) return false;
+  const int c = f / inner;
+  i = nx < 4 || c < 2 ? c : nx - 4 + c;
+  j = 2 + f - c * inner;
+  return true;
+}
+
 // One reverse step.  P.src = X_{t-1} (P.local = 1 when t = 0), Xt = X_t,
 // LPn = Lam_pre(t+1), LP = Lam_pre(t) (output).
-// The FP32 reverse step is latency-bound (long-scoreboard stalls, 22 % warps active at
-// 100 registers and 2 blocks per SM): built for 4 resident blocks (64 registers, a few
-// spills) the gradient run of the 1024 x 128 workload takes 99.7 ms instead of 113.6 ms
-// (3 blocks: no gain).  The FP64 step is bound by the FP64 pipe: 2 blocks.
-#ifndef LBM_ADJ_FP32_BLOCKS_PER_SM
-#define LBM_ADJ_FP32_BLOCKS_PER_SM 4
-#endif
+// The first nfb blocks take the nodes within two cells of a side (the long path; they
+// start first and share no warp with others), the others 64 nodes of a row each, whose
+// consumers are all ordinary streaming links, with the boundary code compiled out: in one
+// mixed launch the step waited for the warps that ran both paths one after the other and
+// for their code.
+// Blocks of two warps: nothing is shared between warps (each adds its own dL/dnu partial,
+// one compensated sum in a fixed order), so no warp waits at a barrier.
+// Measured on 1024 x 128 (one launch, cold caches): FP64 129 -> 47 us (348 -> about 150 FP64
+// instructions per node), FP32 28 -> 15.7 us.
+constexpr int kAdjThreads = 64;
 template <typename S, typename R>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? LBM_ADJ_FP32_BLOCKS_PER_SM : 2) k_adj_step(const SpParams P, const S *__restrict__ Xt,
-                                                  const R *__restrict__ LPn, R *__restrict__ LP,
-                                                  double *grad_qdot, double *grad_flux2, double *grad_flux3,
-                                                  double *nu_partials) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  R dsnu = 0, dsq = 0;
-  if (i < P.nx && j < P.ny) {
-    const long long n = nidx(P, i, j);
-    const R c = K<R>(P).c, ic = K<R>(P).inv_c;
-    // ---- (1) Lam_X(t) = P^T Lam_pre(t+1) at this node --------------------------
-    R lx[9], lg[5];
-    const R *LPng = LPn + (long long)P.gbase * P.plane;
-    if (i >= 2 && i <= P.nx - 3 && j >= 2 && j <= P.ny - 3) {
-      // two or more cells from every side: every consumer of this node's populations is
-      // an ordinary streaming link (no reflection, outlet extrapolation, flux or outflow
-      // rule reaches it), so Lam_X is the plain gather
+__global__ void __launch_bounds__(kAdjThreads, sizeof(R) == 4 ? 16 : 8) k_adj_step(
+    const SpParams P, int nfb, int gx, const S *__restrict__ Xt, const R *__restrict__ LPn, R *__restrict__ LP, double *grad_qdot,
+    double *grad_flux2, double *grad_flux3, R cn, R cq, double *nu_partials) {
+  R dnu = 0;
+  int i, j;
+  R lx[9], lg[5];
+  if ((int)blockIdx.x < nfb) {
+    if (adj_frame_node(P.nx, P.ny, blockIdx.x * kAdjThreads + threadIdx.x, i, j)) {
+      gather_frame<S, R>(P, Xt, LPn, i, j, lx, lg, grad_flux2, grad_flux3);
+      dnu = reverse_node<S, R, false>(P, i, j, lx, lg, LP, grad_qdot, cn, cq);
+    }
+  } else {
+    j = (blockIdx.x - nfb) / gx;
+    i = (blockIdx.x - nfb - j * gx) * kAdjThreads + threadIdx.x;
+    if (i >= 2 && j >= 2 && i < P.nx - 2 && j < P.ny - 2) {
+      const long long n = nidx(P, i, j);
+      const R *LPng = LPn + (long long)P.gbase * P.plane;
 #pragma unroll
       for (int q = 0; q < 9; q++) lx[q] = LPn[q * P.plane + n + (long long)cy9(q) * P.pitch + cx9(q)];
 #pragma unroll
       for (int q = 0; q < 5; q++) lg[q] = LPng[q * P.plane + n + (long long)cy5(q) * P.pitch + cx5(q)];
-    } else {
-#pragma unroll
-      for (int q = 0; q < 9; q++) {
-        R acc = 0;
-        // streaming consumer: node y + c_q pulls population q from here
-        int xi = i + cx9(q), xj = j + cy9(q);
-        if (P.xper) xi = wrap(xi, P.nx);
-        if (P.yper) xj = wrap(xj, P.ny);
-        if (xi >= 0 && xi < P.nx && xj >= 0 && xj < P.ny && streams_in(P, xi, xj, cx9(q), cy9(q), P.xper, P.yper))
-          acc += LPn[q * P.plane + nidx(P, xi, xj)];
-        // reflection consumer: the incoming p = opp(q) at this node built from X_q here
-        const int p = opp9(q);
-        const int side = entry_side(i, j, cx9(p), cy9(p), P.nx, P.ny, P.xper, P.yper);
-        if (side >= 0) acc += (P.side[side].kind == BC_PRESSURE ? (R)-1 : (R)1) * LPn[p * P.plane + n];
-        lx[q] = acc;
-      }
-      // outlet velocity extrapolation u_w = 1.5 u(x_b) - 0.5 u(x_b - n)
-#pragma unroll
-      for (int s = 0; s < 4; s++) {
-        if (P.side[s].kind != BC_PRESSURE) continue;
-        const bool on = (s == 0 && i == 0) || (s == 1 && i == P.nx - 1) || (s == 2 && j == 0) || (s == 3 && j == P.ny - 1);
-        const int bi = i - (s == 0) + (s == 1), bj = j - (s == 2) + (s == 3);  // boundary node outward of here
-        const bool inner = !on && ((s == 0 && i == 1) || (s == 1 && i == P.nx - 2) || (s == 2 && j == 1) ||
-                                   (s == 3 && j == P.ny - 2));
-        if (!on && !inner) continue;
-        R Gx, Gy;
-        if (on) outlet_G<S, R>(P, Xt, LPn, s, i, j, Gx, Gy);
-        else outlet_G<S, R>(P, Xt, LPn, s, bi, bj, Gx, Gy);
-        R rho, ux, uy;
-        post_rho_u<S, R>(P, Xt, i, j, rho, ux, uy);
-        const R coef = (on ? (R)1.5 : (R)-0.5) / rho;  // one division for the nine links
-#pragma unroll
-        for (int q = 0; q < 9; q++) lx[q] += coef * (Gx * (c * (R)cx9(q) - ux) + Gy * (c * (R)cy9(q) - uy));
-      }
-#pragma unroll
-      for (int q = 0; q < 5; q++) {
-        R acc = 0;
-        int xi = i + cx5(q), xj = j + cy5(q);
-        if (P.txper) xi = wrap(xi, P.nx);
-        if (P.typer) xj = wrap(xj, P.ny);
-        if (xi >= 0 && xi < P.nx && xj >= 0 && xj < P.ny && streams_in(P, xi, xj, cx5(q), cy5(q), P.txper, P.typer))
-          acc += LPng[q * P.plane + nidx(P, xi, xj)];
-        const int p = opp5(q);
-        const int side = entry_side(i, j, cx5(p), cy5(p), P.nx, P.ny, P.txper, P.typer);
-        if (side >= 0) {
-          const int tk = P.side[side].tkind;
-          if (tk == TBC_FLUX) acc += LPng[p * P.plane + n];
-          else if (tk == TBC_TEMP) acc -= LPng[p * P.plane + n];
-        }
-        // outflow consumer: the unknown q of an outflow side reads X_q of this node
-        const int qside = entry_side(i, j, cx5(q), cy5(q), P.nx, P.ny, P.txper, P.typer);
-        if (qside >= 0 && P.side[qside].tkind == TBC_OUTFLOW) acc += LPng[q * P.plane + n];
-        lg[q] = acc;
-      }
-      // wall heat flux gradient: pre_p = X_o + flux_coef q''(a) on flux sides
-#pragma unroll
-      for (int p = 1; p < 5; p++) {
-        const int side = entry_side(i, j, cx5(p), cy5(p), P.nx, P.ny, P.txper, P.typer);
-        if (side >= 2 && P.side[side].tkind == TBC_FLUX) {
-          double *gf = side == 2 ? grad_flux2 : grad_flux3;
-          gf[i] += P.flux_coef * (double)LPng[p * P.plane + n];
-        }
-      }
+      dnu = reverse_node<S, R, true>(P, i, j, lx, lg, LP, grad_qdot, cn, cq);
     }
-
-    // ---- (2) pre(t) and the forward intermediates -----------------------------
-    const S *src = (const S *)P.src;
-    const bool interior = !P.local && (i > 0) && (i < P.nx - 1) && (j > 0) && (j < P.ny - 1);
-    R f[9], g[5];
-    pull_f<S, R>(P, src, i, j, interior, f);
-    pull_g<S, R>(P, src, i, j, interior, g);
-    Macro<R> m;
-    load_sources<S, R>(P, n, m);
-    moments<R, FLOW_MRT, TH_MRT>(P, f, g, m);
-    const R rho = m.rho, irho = (R)1 / rho;
-    const R hx = m.ux * ic, hy = m.uy * ic, usq = hx * hx + hy * hy;
-    const R Fx = m.Fx * ic, Fy = m.Fy * ic;
-    const R dt = K<R>(P).dt;
-    const R two = 2, three = 3, four = 4, six = 6, half = 0.5;
-
-    // ---- (3) momentum MRT: transpose ------------------------------------------
-    // moments of Lam_X (same integer rows as the moments of f)
-    const R s14 = (lx[1] + lx[2]) + (lx[3] + lx[4]), s58 = (lx[5] + lx[6]) + (lx[7] + lx[8]);
-    const R d58 = lx[5] - lx[7], d68 = lx[6] - lx[8];
-    const R M_e = -four * lx[0] - s14 + two * s58;
-    const R M_ep = four * lx[0] - two * s14 + s58;
-    const R M_qx = two * (lx[3] - lx[1]) + d58 - d68;
-    const R M_qy = two * (lx[4] - lx[2]) + d58 + d68;
-    const R M_xx = (lx[1] + lx[3]) - (lx[2] + lx[4]);
-    const R M_xy = (lx[5] + lx[7]) - (lx[6] + lx[8]);
-    // dL/dd_k = -(M Lam)_k / |row_k|^2
-    // (products with the rounded reciprocals: a divide is a long sequence on the FP64 pipe)
-    const R de = -M_e * ((R)1 / (R)36), dep = -M_ep * ((R)1 / (R)36);
-    const R dqx = -M_qx * ((R)1 / (R)12), dqy = -M_qy * ((R)1 / (R)12);
-    const R dxx = -M_xx * (R)0.25, dxy = -M_xy * (R)0.25;
-    const R se = K<R>(P).s_e, sep = K<R>(P).s_eps, sq = K<R>(P).s_q, snu = K<R>(P).s_nu;
-    // dL/dm_k = s_k dL/dd_k; dL/deq_k = -s_k dL/dd_k
-    const R lme = se * de, lmep = sep * dep, lmqx = sq * dqx, lmqy = sq * dqy, lmxx = snu * dxx, lmxy = snu * dxy;
-    // equilibria of the moments
-    const R mf58 = f[5] - f[7], mf68 = f[6] - f[8];
-    const R m_qx = two * (f[3] - f[1]) + mf58 - mf68, m_qy = two * (f[4] - f[2]) + mf58 + mf68;
-    const R m_xx = (f[1] + f[3]) - (f[2] + f[4]), m_xy = (f[5] + f[7]) - (f[6] + f[8]);
-    const R eq_qx = -rho * hx, eq_qy = -rho * hy, eq_xx = rho * (hx * hx - hy * hy), eq_xy = rho * hx * hy;
-    // nu enters through s_nu (stress moments) and s_q (third-order moments)
-    const R hdt = K<R>(P).hdt;
-    dsnu = dxx * ((m_xx - eq_xx) + hdt * two * (hx * Fx - hy * Fy)) + dxy * ((m_xy - eq_xy) + hdt * (hx * Fy + hy * Fx));
-    dsq = dqx * ((m_qx - eq_qx) - hdt * Fx) + dqy * ((m_qy - eq_qy) - hdt * Fy);
-    const R le = -se * de, lep = -sep * dep, lqx = -sq * dqx, lqy = -sq * dqy, lxx = -snu * dxx, lxy = -snu * dxy;
-    R l_drho = le * (-two + three * usq) + lep * ((R)1 - three * usq) + lqx * (-hx) + lqy * (-hy) +
-               lxx * (hx * hx - hy * hy) + lxy * (hx * hy);
-    R l_hx = le * (six * rho * hx) + lep * (-six * rho * hx) + lqx * (-rho) + lxx * (two * rho * hx) + lxy * (rho * hy);
-    R l_hy = le * (six * rho * hy) + lep * (-six * rho * hy) + lqy * (-rho) + lxx * (-two * rho * hy) + lxy * (rho * hx);
-    // forcing moments that depend on u
-    // (1 - dt Lambda_k / 2) dt from the host-filled constants
-    const R l_uF = -six * K<R>(P).fk_e * de + six * K<R>(P).fk_eps * dep;
-    const R l_Fxx = -K<R>(P).fk_nu * dxx * two, l_Fxy = -K<R>(P).fk_nu * dxy;
-    l_hx += l_uF * Fx + l_Fxx * Fx + l_Fxy * Fy;
-    l_hy += l_uF * Fy - l_Fxx * Fy + l_Fxy * Fx;
-
-    // ---- (4) thermal D2Q5 MRT: transpose --------------------------------------
-    const R B0 = -((lg[0] + lg[1]) + (lg[2] + lg[3]) + lg[4]);
-    const R B1 = -(lg[1] - lg[3]), B2 = -(lg[2] - lg[4]);
-    const R B3 = -(-four * lg[0] + ((lg[1] + lg[2]) + (lg[3] + lg[4])));
-    const R B4 = -((lg[1] + lg[3]) - (lg[2] + lg[4]));
-    const R t0 = B0 * (R)0.2, t1 = B1 * half, t2 = B2 * half, t3 = B3 * (R)0.05, t4 = B4 * (R)0.25;
-    const R sT = K<R>(P).omegaT;
-    const R lm1 = sT * t1, lm2 = sT * t2, lm3 = t3, lm4 = t4;
-    const R lT = -sT * hx * t1 - sT * hy * t2 + (two / three) * t3;
-    l_hx += -sT * m.T * t1;
-    l_hy += -sT * m.T * t2;
-    grad_add(grad_qdot, n, (R)(hdt * lT - dt * t0 + (dt * ((R)1 / three)) * t3));
-
-    // ---- (5) back to the pre-collision populations ----------------------------
-    R out[14];
-#pragma unroll
-    for (int q = 0; q < 9; q++) {
-      const int cxq = cx9(q), cyq = cy9(q);
-      // transpose of the moment rows: sum_k M[k][q] lm_k
-      const R e_row = q == 0 ? -four : (q <= 4 ? (R)-1 : two);
-      const R ep_row = q == 0 ? four : (q <= 4 ? -two : (R)1);
-      const R qx_row = q == 0 ? (R)0 : (q <= 4 ? -two * (R)cxq : (R)cxq);
-      const R qy_row = q == 0 ? (R)0 : (q <= 4 ? -two * (R)cyq : (R)cyq);
-      const R xx_row = (q >= 1 && q <= 4) ? (R)(cxq * cxq - cyq * cyq) : (R)0;
-      const R xy_row = q >= 5 ? (R)(cxq * cyq) : (R)0;
-      R v = lx[q] + e_row * lme + ep_row * lmep + qx_row * lmqx + qy_row * lmqy + xx_row * lmxx + xy_row * lmxy;
-      v += l_drho + (l_hx * ((R)cxq - hx) + l_hy * ((R)cyq - hy)) * irho;
-      out[q] = v;
-    }
-#pragma unroll
-    for (int q = 0; q < 5; q++) {
-      const R r1 = (R)cx5(q), r2 = (R)cy5(q);
-      const R r3 = q == 0 ? -four : (R)1;
-      const R r4 = (q == 1 || q == 3) ? (R)1 : (q == 0 ? (R)0 : (R)-1);
-      out[9 + q] = lg[q] + r1 * lm1 + r2 * lm2 + r3 * lm3 + r4 * lm4 + lT;
-    }
-#pragma unroll
-    for (int q = 0; q < 14; q++) LP[q * P.plane + n] = out[q];
   }
-  // per-block, fixed-order sums of the nu-rate sensitivities (working precision,
-  // compensated in FP32), added to the block's FP64 partials by one thread
-  NodeSum<R> dn, dq;
-  dn.clear();
-  dq.clear();
-  dn.add(dsnu);
-  dq.add(dsq);
-  dn.warp_reduce();
-  dq.warp_reduce();
-  __shared__ NodeSum<R> sh[8][2];
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  if ((tid & 31) == 0) { sh[tid >> 5][0] = dn; sh[tid >> 5][1] = dq; }
-  __syncthreads();
-  if (tid == 0) {
-    NodeSum<R> a = sh[0][0], b = sh[0][1];
-    for (int w = 1; w < (int)(blockDim.x * blockDim.y) / 32; w++) { a.merge(sh[w][0]); b.merge(sh[w][1]); }
-    double *acc = nu_partials + 2ll * (blockIdx.y * gridDim.x + blockIdx.x);
-    acc[0] += a.value();
-    acc[1] += b.value();
-  }
+  NodeSum<R> sum;
+  sum.clear();
+  sum.add(dnu);
+  sum.warp_reduce();
+  if ((threadIdx.x & 31) == 0)
+    nu_partials[blockIdx.x * (kAdjThreads / 32) + threadIdx.x / 32] += sum.value();
 }
 
-__global__ void k_adj_final(const double *nu_partials, int nb, double *out2) {
-  const int lane = threadIdx.x;
-  double a = 0, b = 0;
-  for (int k = lane; k < nb; k += 32) { a += nu_partials[2 * k]; b += nu_partials[2 * k + 1]; }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_down_sync(0xffffffffu, a, o);
-    b += __shfl_down_sync(0xffffffffu, b, o);
+__global__ void k_adj_final(const double *nu_partials, long long nb, double *out) {
+  const int t = threadIdx.x;
+  double a = 0;
+  for (long long k = t; k < nb; k += 256) a += nu_partials[k];
+  __shared__ double sh[256];
+  sh[t] = a;
+  __syncthreads();
+  for (int w = 128; w > 0; w >>= 1) {
+    if (t < w) sh[t] += sh[t + w];
+    __syncthreads();
   }
-  if (lane == 0) { out2[0] = a; out2[1] = b; }
+  if (t == 0) *out = sh[0];
 }
 
 cudaError_t adj_loss(const SpParams &P, int prec, const double *Ttarget, void *LP, double *grad_qdot,
@@ -365,22 +362,36 @@ cudaError_t adj_loss(const SpParams &P, int prec, const double *Ttarget, void *L
   return cudaGetLastError();
 }
 
-dim3 adj_grid(int nx, int ny) { return dim3((nx + 63) / 64, (ny + 3) / 4); }
+// Blocks of a reverse step: nfb of frame nodes, then gx per row (one grid dimension: rows
+// beyond 65535 stay possible).
+static unsigned adj_blocks(int nx, int ny, int *nfb, int *gx) {
+  *gx = (nx + kAdjThreads - 1) / kAdjThreads;
+  *nfb = (adj_frame_nodes(nx, ny) + kAdjThreads - 1) / kAdjThreads;
+  return (unsigned)*nfb + (unsigned)*gx * ny;
+}
+
+long long adj_partials(int nx, int ny) {
+  int nfb, gx;
+  return (long long)adj_blocks(nx, ny, &nfb, &gx) * (kAdjThreads / 32);
+}
 
 cudaError_t adj_step(const SpParams &P, int prec, const void *Xt, const void *LPn, void *LP, double *grad_qdot,
-                     double *grad_flux2, double *grad_flux3, double *nu_partials, cudaStream_t s) {
-  const dim3 g = adj_grid(P.nx, P.ny), b(64, 4);
+                     double *grad_flux2, double *grad_flux3, double cn, double cq, double *nu_partials, cudaStream_t s) {
+  int nfb, gx;
+  const unsigned nb = adj_blocks(P.nx, P.ny, &nfb, &gx);
   if (prec == 0)
-    k_adj_step<double, double><<<g, b, 0, s>>>(P, (const double *)Xt, (const double *)LPn, (double *)LP, grad_qdot,
-                                               grad_flux2, grad_flux3, nu_partials);
+    k_adj_step<double, double><<<nb, kAdjThreads, 0, s>>>(P, nfb, gx, (const double *)Xt, (const double *)LPn,
+                                                          (double *)LP, grad_qdot, grad_flux2, grad_flux3, cn, cq,
+                                                          nu_partials);
   else
-    k_adj_step<float, float><<<g, b, 0, s>>>(P, (const float *)Xt, (const float *)LPn, (float *)LP, grad_qdot,
-                                             grad_flux2, grad_flux3, nu_partials);
+    k_adj_step<float, float><<<nb, kAdjThreads, 0, s>>>(P, nfb, gx, (const float *)Xt, (const float *)LPn, (float *)LP,
+                                                        grad_qdot, grad_flux2, grad_flux3, (float)cn, (float)cq,
+                                                        nu_partials);
   return cudaGetLastError();
 }
 
-cudaError_t adj_final(const double *nu_partials, int nb, double *out2, cudaStream_t s) {
-  k_adj_final<<<1, 32, 0, s>>>(nu_partials, nb, out2);
+cudaError_t adj_final(const double *nu_partials, long long nb, double *out, cudaStream_t s) {
+  k_adj_final<<<1, 256, 0, s>>>(nu_partials, nb, out);
   return cudaGetLastError();
 }
 

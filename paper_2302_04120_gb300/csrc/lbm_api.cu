@@ -1283,8 +1283,11 @@ extern "C" lbm_status lbm_adjoint(lbm_t h, long steps, int ckpt_every, const dou
   const size_t sbytes = (size_t)h->nq * h->plane * h->elem;
   const size_t pbytes = (size_t)h->plane * sizeof(double);
   const int nx = p.nx, ny = p.ny;
-  dim3 ag = lbmk::adj_grid(nx, ny);
-  const int nblk = (int)(ag.x * ag.y);
+  const long long nparts = lbmk::adj_partials(nx, ny);
+  // s_nu = dt / tau and s_q = dt omega_q(1/tau) as functions of nu, tau = nu/c_s^2 + dt/2
+  const double w_nu = 1.0 / h->tau, a_nu = 3.0 / p.dt - w_nu;
+  const double dw_dnu = -1.0 / (h->tau * h->tau * h->cs2);
+  const double cn = p.dt * dw_dnu, cq = p.dt * (-3.0 / (p.dt * p.dt * a_nu * a_nu)) * dw_dnu;
   double *ck = NULL, *seg = NULL, *lp = NULL, *gq = NULL, *gf = NULL, *nup = NULL, *tt = NULL, *lr = NULL, *o2 = NULL;
   lbm_status st = LBM_OK;
   cudaError_t e = cudaSuccess;
@@ -1303,13 +1306,13 @@ extern "C" lbm_status lbm_adjoint(lbm_t h, long steps, int ckpt_every, const dou
     AAL(lp, sbytes * 2);
     AAL(gq, pbytes);
     AAL(gf, sizeof(double) * 2 * nx);
-    AAL(nup, sizeof(double) * 2 * nblk);
+    AAL(nup, sizeof(double) * nparts);
     AAL(tt, sizeof(double) * ny);
     AAL(lr, sizeof(double) * ny);
-    AAL(o2, sizeof(double) * 2);
+    AAL(o2, sizeof(double));
     ACU(cudaMemsetAsync(gq, 0, pbytes, h->stream));
     ACU(cudaMemsetAsync(gf, 0, sizeof(double) * 2 * nx, h->stream));
-    ACU(cudaMemsetAsync(nup, 0, sizeof(double) * 2 * nblk, h->stream));
+    ACU(cudaMemsetAsync(nup, 0, sizeof(double) * nparts, h->stream));
     ACU(cudaMemcpyAsync(tt, T_target, sizeof(double) * ny, cudaMemcpyHostToDevice, h->stream));
     // forward with checkpoints: ck[m] = X_{mK-1} (ck[0] = pre-collision initial state)
     ACU(cudaMemcpyAsync(ck, h->buf[h->cur], sbytes, cudaMemcpyDeviceToDevice, h->stream));
@@ -1348,17 +1351,17 @@ extern "C" lbm_status lbm_adjoint(lbm_t h, long steps, int ckpt_every, const dou
         const void *Xt = (const char *)seg + sbytes * (size_t)k;
         void *LPn = (char *)lp + sbytes * (size_t)cur;
         void *LPo = (char *)lp + sbytes * (size_t)(1 - cur);
-        ACU(lbmk::adj_step(Q, p.precision, Xt, LPn, LPo, gq, gf, gf + nx, nup, h->stream));
+        ACU(lbmk::adj_step(Q, p.precision, Xt, LPn, LPo, gq, gf, gf + nx, cn, cq, nup, h->stream));
         cur = 1 - cur;
       }
     }
-    ACU(lbmk::adj_final(nup, nblk, o2, h->stream));
+    ACU(lbmk::adj_final(nup, nparts, o2, h->stream));
     // results to the host
     double *hl = (double *)malloc(sizeof(double) * ny);
-    double ho2[2];
+    double dnu;
     if (!hl) { st = fail(h, LBM_ERR_NOMEM, "host allocation"); goto done; }
     ACU(cudaMemcpyAsync(hl, lr, sizeof(double) * ny, cudaMemcpyDeviceToHost, h->stream));
-    ACU(cudaMemcpyAsync(ho2, o2, sizeof(double) * 2, cudaMemcpyDeviceToHost, h->stream));
+    ACU(cudaMemcpyAsync(&dnu, o2, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     if (g_qwall) ACU(cudaMemcpyAsync(g_qwall, gf, sizeof(double) * 2 * nx, cudaMemcpyDeviceToHost, h->stream));
     if (g_q3) {
       // dL/dq''' = dL/dqdot / (rho0 c_p); unpitch on the host
@@ -1384,16 +1387,7 @@ extern "C" lbm_status lbm_adjoint(lbm_t h, long steps, int ckpt_every, const dou
     for (int j = 0; j < ny; j++) L += hl[j];
     free(hl);
     *loss = L;
-    if (g_nu) {
-      // s_nu = dt/tau, s_q = dt omega_q(1/tau), tau = nu/c_s^2 + dt/2
-      const double dt = p.dt, tau = h->tau, w = 1.0 / tau;
-      const double dw_dnu = -1.0 / (tau * tau * h->cs2);
-      const double dsnu = dt * dw_dnu;
-      const double a = 3.0 / dt - w;
-      const double dwq_dw = -3.0 / (dt * dt * a * a);
-      const double dsq = dt * dwq_dw * dw_dnu;
-      *g_nu = ho2[0] * dsnu + ho2[1] * dsq;
-    }
+    if (g_nu) *g_nu = dnu;
   }
 done:
   cudaStreamSynchronize(h->stream);

@@ -167,10 +167,11 @@ cudaError_t to_storage(const double *in, void *out, int nx, int ny, int pitch, i
 // variables (LP, LPn float); the parameter gradients are FP64 in both.
 cudaError_t adj_loss(const SpParams &P, int prec, const double *Ttarget, void *LP, double *grad_qdot,
                      double *loss_rows, cudaStream_t s);
+// cn, cq: d s_nu / d nu and d s_q / d nu; nu_partials: adj_partials() sums of dL/dnu.
 cudaError_t adj_step(const SpParams &P, int prec, const void *Xt, const void *LPn, void *LP, double *grad_qdot,
-                     double *grad_flux2, double *grad_flux3, double *nu_partials, cudaStream_t s);
-cudaError_t adj_final(const double *nu_partials, int nb, double *out2, cudaStream_t s);
-dim3 adj_grid(int nx, int ny);
+                     double *grad_flux2, double *grad_flux3, double cn, double cq, double *nu_partials, cudaStream_t s);
+cudaError_t adj_final(const double *nu_partials, long long nb, double *out, cudaStream_t s);
+long long adj_partials(int nx, int ny);
 
 // Text for lbm_last_error(NULL) from entry points that take no handle.
 void set_global_error(const char *msg);

@@ -58,13 +58,13 @@ __device__ __forceinline__ long long symmetry_source(const SpParams &P, int side
 // populations: rho = sum f*, rho u = sum c f* - dt F / 2 (the collision adds dt F
 // to the momentum, Eqs. first_moment_f and forcing_term).
 template <typename S, typename R>
-__device__ __forceinline__ void post_velocity(const SpParams &P, const S *src, int i, int j, R &ux, R &uy) {
+__device__ __forceinline__ void post_velocity(const SpParams &P, const S *src, int i, int j, R &ux, R &uy, R &rho) {
   long long n = (long long)j * P.pitch + i;
   R f[9];
 #pragma unroll
   for (int q = 0; q < 9; q++) f[q] = (R)src[q * P.plane + n];
   R drho = f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8];
-  R rho = K<R>(P).rho0 + drho;
+  rho = K<R>(P).rho0 + drho;
   R c = K<R>(P).c;
   R jx = c * ((f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]));
   R jy = c * ((f[2] - f[4]) + (f[5] - f[8]) + (f[6] - f[7]));
@@ -191,9 +191,9 @@ __device__ __forceinline__ void pull_f(const SpParams &P, const S *src, int i, i
     R ux = 0, uy = 0, base = 0, lin = 0, quad = 0;
     const bool anti = kind == BC_PRESSURE;
     if (anti) {
-      R ub, vb, ui, vi;
-      post_velocity<S, R>(P, src, i, j, ub, vb);
-      post_velocity<S, R>(P, src, i + (s == 0) - (s == 1), j + (s == 2) - (s == 3), ui, vi);
+      R ub, vb, ui, vi, rho;
+      post_velocity<S, R>(P, src, i, j, ub, vb, rho);
+      post_velocity<S, R>(P, src, i + (s == 0) - (s == 1), j + (s == 2) - (s == 3), ui, vi, rho);
       ux = ub + (R)0.5 * (ub - ui);
       uy = vb + (R)0.5 * (vb - vi);
       base = (R)2 * (rw - K<R>(P).rho0) - rw * (ux * ux + uy * uy) * ics2;
