@@ -261,6 +261,7 @@ static lbmk::MpParams mp_params(const lbm_t h, int from_buf) {
   const lbm_params &p = h->p;
   P.nx = p.nx; P.ny = p.ny; P.pitch = h->pitch; P.plane = h->plane;
   P.c = h->c; P.cs2 = h->cs2; P.dt = p.dt; P.dx = p.dx;
+  P.inv_c = 1.0 / h->c;
   P.rho_l = p.rho_l; P.rho_g = p.rho_g; P.nu_l = p.nu_l; P.nu_g = p.nu_g;
   P.kappa = 1.5 * p.sigma * p.W;   // kappa = 3 sigma W / 2
   P.beta = 12.0 * p.sigma / p.W;   // beta = 12 sigma / W

@@ -21,7 +21,7 @@ struct MpConst {
 struct MpParams {
   int nx, ny, pitch;
   long long plane;
-  double c, cs2, dt, dx;
+  double c, cs2, dt, dx, inv_c;
   double rho_l, rho_g, nu_l, nu_g;
   double kappa, beta, W, tauphi;
   int nu_rule, z_mrt, qy_literal;
