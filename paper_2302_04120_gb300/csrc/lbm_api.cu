@@ -191,8 +191,10 @@ static SpParams sp_params(const lbm_t h, int from_buf) {
     P.side[s].kind = h->bc[s];
     P.side[s].tkind = h->tbc[s];
     P.side[s].rho_w = h->rho_w[s];
-    P.side[s].uw = h->d_uw[s];
-    P.side[s].tw = h->d_tw[s];
+    // no array for walls at rest and adiabatic sides: the frame's warps, the critical path
+    // of a small grid, then skip its loads and the links' velocity terms
+    P.side[s].uw = h->uw_zero[s] ? NULL : h->d_uw[s];
+    P.side[s].tw = h->tw_zero[s] ? NULL : h->d_tw[s];
   }
   P.c = h->c; P.cs2 = h->cs2; P.dt = p.dt; P.dx = p.dx;
   P.rho0 = p.rho0; P.T0 = p.T0;

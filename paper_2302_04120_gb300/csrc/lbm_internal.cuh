@@ -12,8 +12,8 @@ struct DevSide {
   int kind;          // LBM_BC_*
   int tkind;         // LBM_TBC_*
   double rho_w;      // boundary density of Eqs. BB_vel / anti_BB_vel
-  const double *uw;  // 2*len: u_x then u_y at each boundary node
-  const double *tw;  // len: q'' (FLUX) or T_w (TEMP)
+  const double *uw;  // 2*len: u_x then u_y at each boundary node; NULL: zero
+  const double *tw;  // len: q'' (FLUX) or T_w (TEMP); NULL: zero
 };
 
 // Constants of a single-phase solve in the working precision R, filled on the host:

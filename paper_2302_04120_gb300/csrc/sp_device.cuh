@@ -200,11 +200,10 @@ __device__ __forceinline__ void pull_f(const SpParams &P, const S *src, int i, i
       quad = rw * ics2 * ics2;
     } else {
       const double *uw = P.side[s].uw;
-      if (uw) {
-        const int a = along(s, i, j);
-        ux = (R)uw[a];
-        uy = (R)uw[side_len(P, s) + a];
-      }
+      if (!uw) continue;  // at rest: f_q = f_o*
+      const int a = along(s, i, j);
+      ux = (R)uw[a];
+      uy = (R)uw[side_len(P, s) + a];
       lin = (R)2 * rw * ics2;
     }
 #pragma unroll
