@@ -37,6 +37,7 @@ struct lbm_s {
   double *h_stage[4];        // pinned staging of the boundary arrays, one slot per side
   cudaEvent_t stage_done[4];  // the slot's last upload has been consumed
   int uw_zero[4], tw_zero[4];  // the device array holds zeros (no upload since the last fill)
+  int uw_used[4], tw_used[4];  // the device array has held values
   // sources (storage precision, pitched)
   void *d_qdot, *d_force;
   // lagged heat sink (lbm_set_lagged_sink): qdot = qbase - conv (T(t - dt) - T_inf); the
@@ -172,10 +173,21 @@ static void fill_const(const SpParams &P, lbmk::SpConst<R> &k) {
   for (int s = 0; s < 4; s++) k.rho_w[s] = (R)P.side[s].rho_w;
 }
 
-static SpParams sp_params(const lbm_t h, int from_buf) {
+// Whether the caller is capturing the solve's stream into a graph of its own.
+static bool recording(const lbm_t h) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream while another one is captured: not this one
+    return false;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
+static SpParams sp_params(const lbm_t h, int from_buf, bool arrays = false) {
   SpParams P;
   memset(&P, 0, sizeof(P));
   const lbm_params &p = h->p;
+  arrays = arrays || recording(h);
   P.nx = p.nx; P.ny = p.ny; P.pitch = h->pitch; P.plane = h->plane;
   P.xper = axis_periodic(h, 0, 0); P.yper = axis_periodic(h, 1, 0);
   P.txper = axis_periodic(h, 0, 1); P.typer = axis_periodic(h, 1, 1);
@@ -192,9 +204,12 @@ static SpParams sp_params(const lbm_t h, int from_buf) {
     P.side[s].tkind = h->tbc[s];
     P.side[s].rho_w = h->rho_w[s];
     // no array for walls at rest and adiabatic sides: the frame's warps, the critical path
-    // of a small grid, then skip its loads and the links' velocity terms
-    P.side[s].uw = h->uw_zero[s] ? NULL : h->d_uw[s];
-    P.side[s].tw = h->tw_zero[s] ? NULL : h->d_tw[s];
+    // of a small grid, then skip its loads and the links' velocity terms.  A side that has
+    // held values keeps its array (a wall heated now and then keeps one parameter block and
+    // its captured steps); a batch's tables and launches that the caller captures name every
+    // array (arrays), so that a replay sees what was uploaded since
+    P.side[s].uw = h->uw_used[s] || arrays ? h->d_uw[s] : NULL;
+    P.side[s].tw = h->tw_used[s] || arrays ? h->d_tw[s] : NULL;
   }
   P.c = h->c; P.cs2 = h->cs2; P.dt = p.dt; P.dx = p.dx;
   P.rho0 = p.rho0; P.T0 = p.T0;
@@ -470,6 +485,7 @@ extern "C" lbm_status lbm_set_bc(lbm_t h, int side, int kind, const double *uw, 
     memcpy(st, uw, sizeof(double) * 2 * len);
     CU(h, cudaMemcpyAsync(h->d_uw[side], st, sizeof(double) * 2 * len, cudaMemcpyHostToDevice, h->stream));
     h->uw_zero[side] = 0;
+    h->uw_used[side] = 1;
   } else if (!h->uw_zero[side]) {
     CU(h, cudaMemsetAsync(h->d_uw[side], 0, sizeof(double) * 2 * len, h->stream));
     h->uw_zero[side] = 1;
@@ -478,6 +494,7 @@ extern "C" lbm_status lbm_set_bc(lbm_t h, int side, int kind, const double *uw, 
     memcpy(st + 2 * len, tw, sizeof(double) * len);
     CU(h, cudaMemcpyAsync(h->d_tw[side], st + 2 * len, sizeof(double) * len, cudaMemcpyHostToDevice, h->stream));
     h->tw_zero[side] = 0;
+    h->tw_used[side] = 1;
   } else if (!h->tw_zero[side]) {
     CU(h, cudaMemsetAsync(h->d_tw[side], 0, sizeof(double) * len, h->stream));
     h->tw_zero[side] = 1;
@@ -1117,10 +1134,10 @@ static lbm_status batch_tables(lbm_batch_t b, int *cur, int *pre) {
     lbm_t h = b->ch[k];
     const int save = h->pre;
     h->pre = 0;
-    tmp[k] = sp_params(h, 0);
-    tmp[b->n + k] = sp_params(h, 1);
+    tmp[k] = sp_params(h, 0, true);
+    tmp[b->n + k] = sp_params(h, 1, true);
     h->pre = 1;
-    tmp[2 * b->n + k] = sp_params(h, c0);
+    tmp[2 * b->n + k] = sp_params(h, c0, true);
     h->pre = save;
   }
   if (!b->tab_valid || memcmp(tmp, b->h_tab, 3 * (size_t)b->n * sizeof(SpParams)) != 0) {
@@ -1482,7 +1499,7 @@ extern "C" lbm_status lbm_autotune(lbm_t h, int out_block[2]) {
   // candidates: grid launches of 32..256 threads, then TMA launches
   int cands[64][4];
   int nc = 0;
-  static const int shapes[][2] = {{32, 2}, {32, 4}, {32, 8}, {64, 1}, {64, 2}, {64, 4}, {128, 1}, {128, 2}, {256, 1}};
+  static const int shapes[][2] = {{32, 1}, {32, 2}, {32, 4}, {32, 8}, {64, 1}, {64, 2}, {64, 4}, {128, 1}, {128, 2}, {256, 1}};
   for (int kind = LBM_LAUNCH_GRID; kind <= LBM_LAUNCH_GRID_OCC; kind += LBM_LAUNCH_GRID_OCC - LBM_LAUNCH_GRID)
     for (const auto &sh : shapes) {
       cands[nc][0] = kind; cands[nc][1] = sh[0]; cands[nc][2] = sh[1]; cands[nc][3] = 0;
