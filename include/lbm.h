@@ -358,9 +358,11 @@ void lbm_destroy(lbm_t h);
 /*
  * Batched solves: many independent single-phase channels of uneven size advanced
  * together, one kernel launch per time step over a flattened (channel, tile) list,
- * replayed from a CUDA graph.  Each channel is an ordinary lbm_t owned by the batch:
- * set its boundaries, sources and initial fields and read its moments with the calls
- * above (lbm_batch_channel), but advance it only with lbm_batch_step.
+ * replayed from a CUDA graph; in FP32, where a call takes several steps, group by group
+ * (as many channels as stay in L2, each group all the call's steps).  Each channel is an
+ * ordinary lbm_t owned by the batch: set its boundaries, sources and initial fields and
+ * read its moments with the calls above (lbm_batch_channel), but advance it only with
+ * lbm_batch_step.
  *  lbm_batch_create  n parameter blocks (same precision, lattices and operators; single
  *                    phase); stream NULL = a private non-blocking stream (graph capture
  *                    cannot use the legacy default stream).  Errors as lbm_create.

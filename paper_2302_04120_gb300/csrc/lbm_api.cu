@@ -979,6 +979,9 @@ struct lbm_batch_s {
   int4 *d_tiles;
   int ntiles, tiles_bx, tiles_by;
   int bx, by, grid;       // launch configuration (autotuned or set)
+  int *order, *first;     // channels group by group; group g is order[first[g]] .. order[first[g + 1] - 1]
+  int *tile0;             // its entries are tiles tile0[g] .. tile0[g + 1] - 1
+  int ngroups;
   cudaGraph_t graph;
   cudaGraphExec_t exec;   // two steps: parity 0 then parity 1
   char err[512];
@@ -1015,10 +1018,53 @@ extern "C" void lbm_batch_destroy(lbm_batch_t b) {
   for (int k = 0; k < b->n; k++) lbm_destroy(b->ch[k]);
   free(b->ch);
   free(b->h_tab);
+  free(b->order);
+  free(b->first);
+  free(b->tile0);
   cudaFree(b->d_tab);
   cudaFree(b->d_tiles);
   if (b->own_stream) cudaStreamDestroy(b->stream);
   free(b);
+}
+
+// How a batch of FP32 channels is split (kGroupMinSteps: fewer steps of one call reuse too
+// little).  Measured on GB300, MRT + D2Q5 MRT channels, billions of node updates per second,
+// back-to-back steps of one channel of n thousand nodes (state_bytes MB) as a single solve and
+// as one batched launch per step:
+//   66 (7 MB): 17 and 6;  131 (15 MB): 30 and 11;  262 (29 MB): 51 and 20;  524 (59 MB): 75
+//   and 32;  768 (86 MB): 76 and 39;  1024 (115 MB): 60 and 42;  3200 (358 MB): 59 and 49.
+// So a channel of more than 16 MB runs as a single solve (parameters in constant memory, the
+// frame spread over the SMs); smaller ones share launches, as many as fill 60 MB (48 uneven
+// channels, 48 steps: 25.4 ms with 60 MB, 25.7 with 80, 26.1 with 40 or 110, 26.7 with one
+// launch per step over all, in a first form that took single solves from half of that size).
+constexpr double kAloneBytes = 16e6, kGroupBytes = 60e6;
+constexpr long kGroupMinSteps = 4;
+
+static double state_bytes(const lbm_t h) { return 2.0 * h->nq * h->plane * h->elem; }
+static bool batch_alone(const lbm_t h) { return state_bytes(h) > kAloneBytes; }
+
+// Groups: every channel alone that can be, the others in order of index
+// as long as their state fits.
+static void batch_groups(lbm_batch_t b) {
+  int at = 0;
+  b->ngroups = 0;
+  for (int k = 0; k < b->n; k++)
+    if (batch_alone(b->ch[k])) {
+      b->first[b->ngroups++] = at;
+      b->order[at++] = k;
+    }
+  double held = 2.0 * kGroupBytes;
+  for (int k = 0; k < b->n; k++) {
+    if (batch_alone(b->ch[k])) continue;
+    const double need = state_bytes(b->ch[k]);
+    if (held + need > kGroupBytes) {
+      b->first[b->ngroups++] = at;
+      held = 0.0;
+    }
+    held += need;
+    b->order[at++] = k;
+  }
+  b->first[b->ngroups] = at;
 }
 
 extern "C" lbm_status lbm_batch_create(const lbm_params *params, int n, void *stream, lbm_batch_t *out) {
@@ -1037,7 +1083,14 @@ extern "C" lbm_status lbm_batch_create(const lbm_params *params, int n, void *st
   b->n = n;
   b->ch = (lbm_t *)calloc(n, sizeof(lbm_t));
   b->h_tab = (SpParams *)calloc(3 * (size_t)n, sizeof(SpParams));
-  if (!b->ch || !b->h_tab) { lbm_batch_destroy(b); return bfail(NULL, LBM_ERR_NOMEM, "host allocation failed"); }
+  b->order = (int *)malloc(n * sizeof(int));
+  b->first = (int *)malloc((n + 1) * sizeof(int));
+  b->tile0 = (int *)malloc((n + 1) * sizeof(int));
+  if (!b->ch || !b->h_tab || !b->order || !b->first || !b->tile0) {
+    b->n = b->ch ? n : 0;
+    lbm_batch_destroy(b);
+    return bfail(NULL, LBM_ERR_NOMEM, "host allocation failed");
+  }
   if (stream) {
     b->stream = (cudaStream_t)stream;
   } else {  // graph capture needs a stream other than the legacy default one
@@ -1056,6 +1109,7 @@ extern "C" lbm_status lbm_batch_create(const lbm_params *params, int n, void *st
       return bfail(NULL, st, "%s", msg);
     }
   }
+  batch_groups(b);
   b->prec = params[0].precision;
   sp_kinds(b->ch[0], &b->flow, &b->th);
   if (cudaMalloc(&b->d_tab, 3 * (size_t)n * sizeof(SpParams)) != cudaSuccess) {
@@ -1080,8 +1134,8 @@ extern "C" lbm_t lbm_batch_channel(lbm_batch_t b, int k) {
 
 extern "C" int lbm_batch_size(lbm_batch_t b) { return b ? b->n : 0; }
 
-// (Re)build the entry list for a tile shape: every channel's boundary frame in
-// chunks of bx*by nodes first (the longest-running nodes start first), then the
+// (Re)build the entry list for a tile shape: group by group, every channel's boundary
+// frame in chunks of bx*by nodes first (the longest-running nodes start first), then the
 // interior tiles.
 static lbm_status batch_tiles(lbm_batch_t b, int bx, int by) {
   if (b->d_tiles && b->tiles_bx == bx && b->tiles_by == by) return LBM_OK;
@@ -1096,15 +1150,19 @@ static lbm_status batch_tiles(lbm_batch_t b, int bx, int by) {
   int4 *h = (int4 *)malloc(sizeof(int4) * (size_t)total);
   if (!h) return bfail(b, LBM_ERR_NOMEM, "host allocation failed");
   long long t = 0;
-  for (int k = 0; k < b->n; k++) {
-    const int nf = lbmk::frame_nodes(b->ch[k]->p.nx, b->ch[k]->p.ny);
-    for (int f0 = 0; f0 < nf; f0 += chunk) h[t++] = make_int4(k, f0, 0, 1);
+  for (int g = 0; g < b->ngroups; g++) {
+    b->tile0[g] = (int)t;
+    for (int o = b->first[g]; o < b->first[g + 1]; o++) {
+      const int k = b->order[o], nf = lbmk::frame_nodes(b->ch[k]->p.nx, b->ch[k]->p.ny);
+      for (int f0 = 0; f0 < nf; f0 += chunk) h[t++] = make_int4(k, f0, 0, 1);
+    }
+    for (int o = b->first[g]; o < b->first[g + 1]; o++) {
+      const int k = b->order[o], nx = b->ch[k]->p.nx, ny = b->ch[k]->p.ny;
+      for (int y0 = 0; y0 < ny; y0 += by)
+        for (int x0 = 0; x0 < nx; x0 += bx) h[t++] = make_int4(k, x0, y0, 0);
+    }
   }
-  for (int k = 0; k < b->n; k++) {
-    const int nx = b->ch[k]->p.nx, ny = b->ch[k]->p.ny;
-    for (int y0 = 0; y0 < ny; y0 += by)
-      for (int x0 = 0; x0 < nx; x0 += bx) h[t++] = make_int4(k, x0, y0, 0);
-  }
+  b->tile0[b->ngroups] = (int)t;
   cudaStreamSynchronize(b->stream);
   cudaFree(b->d_tiles);
   b->d_tiles = NULL;
@@ -1197,6 +1255,29 @@ extern "C" lbm_status lbm_batch_step(lbm_batch_t b, long n) {
     batch_advance(b, 1);
     n--;
     cur = 1 - cur;
+  }
+  // FP32: each group takes all n steps before the next one, so that its state stays in L2
+  // (one launch per step over all channels streams every state from HBM each step).  FP64
+  // steps are bound by the FP64 pipe and keep one launch per step.
+  if (b->prec != LBM_FP64 && (b->ngroups > 1 || batch_alone(b->ch[0])) && n >= kGroupMinSteps) {
+    for (int g = 0; g < b->ngroups; g++) {
+      lbm_t h = b->ch[b->order[b->first[g]]];
+      if (batch_alone(h) && h->launch_kind != LBM_LAUNCH_TMA) {
+        st = advance(h, n);
+        if (st != LBM_OK) return bfail(b, st, "channel %d: %s", b->order[b->first[g]], h->err);
+        continue;
+      }
+      const int nt = b->tile0[g + 1] - b->tile0[g];
+      for (long s = 0; s < n; s++)
+        BCU(b, lbmk::sp_batch_step(b->d_tab + (size_t)((cur + s) & 1) * b->n, b->d_tiles + b->tile0[g], nt, b->prec, b->flow,
+                                   b->th, dim3(b->bx, b->by), b->grid < nt ? b->grid : nt, b->stream));
+      for (int o = b->first[g]; o < b->first[g + 1]; o++) {
+        lbm_t c = b->ch[b->order[o]];
+        c->cur = (int)((c->cur + n) & 1);
+        c->steps += n;
+      }
+    }
+    return LBM_OK;
   }
   if (n > 0 && cur == 1) {  // align to parity 0 for the two-step graph
     BCU(b, batch_launch(b, b->d_tab + b->n));
