@@ -49,7 +49,7 @@ struct lbm_s {
   int max_blocks;
   double *d_out4;  // 4 integrals, the step kernels' error flag (an int in slot 4) and the
                    // integrals' block counter (an unsigned in slot 5, zero between calls)
-  double *h_out4;  // pinned, 5 doubles
+  double *h_out4;  // pinned, 5 doubles: integrals and flag, written by the reducing kernel
   dim3 block;
   // single-phase step launch: LBM_LAUNCH_GRID (one node per thread, `block`) or
   // LBM_LAUNCH_TMA (persistent CTAs of 32 x tma_ty threads, boxes staged by TMA)
@@ -483,7 +483,6 @@ extern "C" lbm_status lbm_set_bc(lbm_t h, int side, int kind, const double *uw, 
   if (uw || tw) CU(h, cudaEventSynchronize(h->stage_done[side]));
   if (uw) {
     memcpy(st, uw, sizeof(double) * 2 * len);
-    CU(h, cudaMemcpyAsync(h->d_uw[side], st, sizeof(double) * 2 * len, cudaMemcpyHostToDevice, h->stream));
     h->uw_zero[side] = 0;
     h->uw_used[side] = 1;
   } else if (!h->uw_zero[side]) {
@@ -492,14 +491,17 @@ extern "C" lbm_status lbm_set_bc(lbm_t h, int side, int kind, const double *uw, 
   }
   if (tw) {
     memcpy(st + 2 * len, tw, sizeof(double) * len);
-    CU(h, cudaMemcpyAsync(h->d_tw[side], st + 2 * len, sizeof(double) * len, cudaMemcpyHostToDevice, h->stream));
     h->tw_zero[side] = 0;
     h->tw_used[side] = 1;
   } else if (!h->tw_zero[side]) {
     CU(h, cudaMemsetAsync(h->d_tw[side], 0, sizeof(double) * len, h->stream));
     h->tw_zero[side] = 1;
   }
-  if (uw || tw) CU(h, cudaEventRecord(h->stage_done[side], h->stream));
+  if (uw || tw) {
+    CU(h, lbmk::upload_side(st, h->d_uw[side], uw ? 2ll * len : 0, h->d_tw[side], tw ? len : 0, 2ll * len,
+                             h->stream));
+    CU(h, cudaEventRecord(h->stage_done[side], h->stream));
+  }
   return LBM_OK;
 }
 
@@ -893,16 +895,15 @@ extern "C" lbm_status lbm_integrals(lbm_t h, double out[4]) {
   cudaError_t e;
   if (two_phase(h)) {
     lbmk::MpParams P = mp_params(h, h->cur);
-    e = lbmk::mp_integrals(P, h->p.precision, h->d_partials, h->max_blocks, h->d_out4, h->stream);
+    e = lbmk::mp_integrals(P, h->p.precision, h->d_partials, h->max_blocks, h->h_out4, h->d_out4 + 4, h->stream);
   } else {
     int flow, th;
     sp_kinds(h, &flow, &th);
     SpParams P = sp_params(h, h->cur);
-    e = lbmk::sp_integrals(P, h->p.precision, flow, th, h->d_partials, h->max_blocks, h->d_out4,
+    e = lbmk::sp_integrals(P, h->p.precision, flow, th, h->d_partials, h->max_blocks, h->h_out4, h->d_out4 + 4,
                            (unsigned *)(h->d_out4 + 5), h->stream);
   }
   if (e != cudaSuccess) return fail(h, LBM_ERR_CUDA, "integrals launch: %s", cudaGetErrorString(e));
-  CU(h, cudaMemcpyAsync(h->h_out4, h->d_out4, 5 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CU(h, cudaStreamSynchronize(h->stream));
   memcpy(out, h->h_out4, 4 * sizeof(double));
   int flag;

@@ -155,9 +155,18 @@ cudaError_t sp_moments(const SpParams &P, int prec, int flow, int th, unsigned m
                        double *out, cudaStream_t s);
 // Per-block partial integrals (4 doubles per block) then a fixed-order final reduction.
 // counter: a device unsigned that is 0 on entry; the kernel's last block resets it.
+// out5: the four integrals and the word at flag (the step kernels' error flag); pinned host
+// memory, so that no copy stands between the kernel and the caller's read.
 cudaError_t sp_integrals(const SpParams &P, int prec, int flow, int th, double *partials,
-                         int max_blocks, double *out4, unsigned *counter, cudaStream_t s);
+                         int max_blocks, double *out5, const double *flag, unsigned *counter, cudaStream_t s);
 int sp_integral_blocks(int nx, int ny);
+
+// Boundary arrays of one side from its pinned staging slot (uw first, tw at tw_at; nu and nt
+// values of them).  A kernel that reads the slot over the link, not a copy: for a few KB the
+// copy engine's hand-overs are the cost.  A pass of two uploads, one step, integrals and a
+// field on 2048 x 256 FP32: 114 -> 101 us, with the integrals written to pinned memory.
+cudaError_t upload_side(const double *stage, double *uw, long long nu, double *tw, long long nt,
+                          long long tw_at, cudaStream_t s);
 
 // Convert nx*ny double planes into pitched storage planes (sources, forces).
 cudaError_t to_storage(const double *in, void *out, int nx, int ny, int pitch, int nplanes,

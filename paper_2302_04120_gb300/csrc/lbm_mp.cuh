@@ -48,7 +48,7 @@ cudaError_t mp_step(const MpParams &P, int prec, cudaStream_t s);
 cudaError_t mp_init(const MpParams &P, int prec, const double *phi0, const double *ux0, const double *uy0,
                     const double *p0, cudaStream_t s);
 cudaError_t mp_moments(const MpParams &P, int prec, unsigned mask, double *out, cudaStream_t s);
-cudaError_t mp_integrals(const MpParams &P, int prec, double *partials, int max_blocks, double *out4,
+cudaError_t mp_integrals(const MpParams &P, int prec, double *partials, int max_blocks, double *out5, const double *flag,
                          cudaStream_t s);
 int mp_integral_blocks(int nx, int ny);
 

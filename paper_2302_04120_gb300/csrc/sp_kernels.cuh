@@ -283,7 +283,7 @@ __device__ __forceinline__ void block_partials(Part<R> a, Part<R> *out) {
 // healthy nodes of (rho - rho0)) dx^2, max |u| = sqrt(max |u|^2).
 template <typename R>
 __device__ __forceinline__ void final_reduce(const Part<R> *parts, int nb, double n_rho0, double rho0, double area,
-                                             double *out4) {
+                                             double *out5, const double *flag) {
   const int t = threadIdx.y * blockDim.x + threadIdx.x;
   Part<R> a;
   a.clear();
@@ -297,10 +297,11 @@ __device__ __forceinline__ void final_reduce(const Part<R> *parts, int nb, doubl
   }
   if (t == 0) {
     const double bad = (double)sh[0].bad;
-    out4[0] = (n_rho0 - bad * rho0 + sh[0].s.value()) * area;
-    out4[1] = 0.0;
-    out4[2] = sqrt((double)sh[0].u2);
-    out4[3] = bad;
+    out5[0] = (n_rho0 - bad * rho0 + sh[0].s.value()) * area;
+    out5[1] = 0.0;
+    out5[2] = sqrt((double)sh[0].u2);
+    out5[3] = bad;
+    out5[4] = *flag;
   }
 }
 
@@ -334,7 +335,7 @@ __device__ __forceinline__ void integrate_node(const SpParams &P, int i, int j, 
 
 template <int PREC, int FLOW, int TH, bool SYM>
 __global__ void __launch_bounds__(256, 3) k_integrals(const SpParams P, int steps, int fy, double *partials,
-                                                      double n_rho0, double area, double *out4, unsigned *counter) {
+                                                      double n_rho0, double area, double *out5, const double *flag, unsigned *counter) {
   // n_rho0 = N rho0 of the whole grid; final_reduce removes rho0 per bad node
   typedef typename Prec<PREC>::S S;
   typedef typename Prec<PREC>::R R;
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__(256, 3) k_integrals(const SpParams P, int step
   __syncthreads();
   if (last) {
     __threadfence();
-    final_reduce<R>(parts, (int)nb, n_rho0, P.rho0, area, out4);
+    final_reduce<R>(parts, (int)nb, n_rho0, P.rho0, area, out5, flag);
     if (threadIdx.x == 0 && threadIdx.y == 0) *counter = 0u;
   }
 }
@@ -439,16 +440,16 @@ cudaError_t SpOps<PREC, FLOW, TH>::moments(const SpParams &P, unsigned mask, dou
 }
 
 template <int PREC, int FLOW, int TH>
-cudaError_t SpOps<PREC, FLOW, TH>::integrals(const SpParams &P, double *partials, double *out4, unsigned *counter,
-                                             cudaStream_t s) {
+cudaError_t SpOps<PREC, FLOW, TH>::integrals(const SpParams &P, double *partials, double *out5, const double *flag,
+                                             unsigned *counter, cudaStream_t s) {
   const dim3 block(kRedBX, kRedBY);
   const double n_rho0 = (double)P.nx * P.ny * P.rho0, area = P.dx * P.dx;
   int steps, fy;
   const dim3 grid = integral_grid(P.nx, P.ny, &steps, &fy);
   if (P.sym)
-    k_integrals<PREC, FLOW, TH, true><<<grid, block, 0, s>>>(P, steps, fy, partials, n_rho0, area, out4, counter);
+    k_integrals<PREC, FLOW, TH, true><<<grid, block, 0, s>>>(P, steps, fy, partials, n_rho0, area, out5, flag, counter);
   else
-    k_integrals<PREC, FLOW, TH, false><<<grid, block, 0, s>>>(P, steps, fy, partials, n_rho0, area, out4, counter);
+    k_integrals<PREC, FLOW, TH, false><<<grid, block, 0, s>>>(P, steps, fy, partials, n_rho0, area, out5, flag, counter);
   return cudaGetLastError();
 }
 

@@ -25,7 +25,7 @@ struct SpOps {
   static cudaError_t init(const SpParams &P, const double *a, const double *ux, const double *uy, const double *b,
                           dim3 block, cudaStream_t s);
   static cudaError_t moments(const SpParams &P, unsigned mask, double *out, cudaStream_t s);
-  static cudaError_t integrals(const SpParams &P, double *partials, double *out4, unsigned *counter,
+  static cudaError_t integrals(const SpParams &P, double *partials, double *out5, const double *flag, unsigned *counter,
                                cudaStream_t s);
 };
 

@@ -493,7 +493,7 @@ k_mp_collide(const MpParams P, unsigned mask, double *out) {
   if (MODE == MODE_INTEGRALS) reduce4_block(red, out + 4ll * (blockIdx.y * gridDim.x + blockIdx.x));
 }
 
-__global__ void k_mp_final(const double *partials, int nb, double *out4) {
+__global__ void k_mp_final(const double *partials, int nb, double *out5, const double *flag) {
   const int lane = threadIdx.x;
   double v[4] = {0.0, 0.0, 0.0, 0.0};
   for (int b = lane; b < nb; b += 32) {
@@ -509,7 +509,7 @@ __global__ void k_mp_final(const double *partials, int nb, double *out4) {
     v[2] = fmax(v[2], __shfl_down_sync(0xffffffffu, v[2], o));
     v[3] += __shfl_down_sync(0xffffffffu, v[3], o);
   }
-  if (lane == 0) { out4[0] = v[0]; out4[1] = v[1]; out4[2] = v[2]; out4[3] = v[3]; }
+  if (lane == 0) { out5[0] = v[0]; out5[1] = v[1]; out5[2] = v[2]; out5[3] = v[3]; out5[4] = *flag; }
 }
 
 // Equilibria of the given fields (Eqs. heq_liang, zeq_liang, s_i_Liang) as the
@@ -597,12 +597,13 @@ cudaError_t mp_moments(const MpParams &P, int prec, unsigned mask, double *out, 
   return cudaGetLastError();
 }
 
-cudaError_t mp_integrals(const MpParams &P, int prec, double *partials, int max_blocks, double *out4, cudaStream_t s) {
+cudaError_t mp_integrals(const MpParams &P, int prec, double *partials, int max_blocks, double *out5, const double *flag,
+                         cudaStream_t s) {
   const int nb = mp_integral_blocks(P.nx, P.ny);
   if (nb > max_blocks) return cudaErrorInvalidValue;
   if (prec == 0) launch_collide<0, MODE_INTEGRALS>(P, 0u, partials, s);
   else launch_collide<1, MODE_INTEGRALS>(P, 0u, partials, s);
-  k_mp_final<<<1, 32, 0, s>>>(partials, nb, out4);
+  k_mp_final<<<1, 32, 0, s>>>(partials, nb, out5, flag);
   return cudaGetLastError();
 }
 

@@ -94,11 +94,11 @@ int sp_integral_blocks(int nx, int ny) {
 }
 
 cudaError_t sp_integrals(const SpParams &P, int prec, int flow, int th, double *partials, int max_blocks,
-                         double *out4, unsigned *counter, cudaStream_t s) {
+                         double *out5, const double *flag, unsigned *counter, cudaStream_t s) {
   int steps, fy;
   dim3 grid = integral_grid(P.nx, P.ny, &steps, &fy);
   if ((int)(grid.x * grid.y) > max_blocks) return cudaErrorInvalidValue;
-#define LBM_SP_BODY(A, B, C) return SpOps<A, B, C>::integrals(P, partials, out4, counter, s)
+#define LBM_SP_BODY(A, B, C) return SpOps<A, B, C>::integrals(P, partials, out5, flag, counter, s)
   LBM_SP_COMBOS(LBM_SP_CASE)
 #undef LBM_SP_BODY
   return cudaErrorInvalidValue;
@@ -122,6 +122,21 @@ cudaError_t to_storage(const double *in, void *out, int nx, int ny, int pitch, i
   dim3 b(64, 4), g = grid_for(nx, ny, b);
   if (prec == 0) k_to_storage<double><<<g, b, 0, s>>>(in, (double *)out, nx, ny, pitch, nplanes, plane, scale);
   else k_to_storage<float><<<g, b, 0, s>>>(in, (float *)out, nx, ny, pitch, nplanes, plane, scale);
+  return cudaGetLastError();
+}
+
+__global__ void k_upload_side(const double *stage, double *uw, long long nu, double *tw, long long nt,
+                          long long tw_at) {
+  for (long long k = blockIdx.x * blockDim.x + threadIdx.x; k < nu + nt; k += gridDim.x * blockDim.x) {
+    if (k < nu) uw[k] = stage[k];
+    else tw[k - nu] = stage[tw_at + k - nu];
+  }
+}
+
+cudaError_t upload_side(const double *stage, double *uw, long long nu, double *tw, long long nt,
+                          long long tw_at, cudaStream_t s) {
+  const long long blocks = (nu + nt + 255) / 256;
+  k_upload_side<<<(unsigned)(blocks < 64 ? blocks : 64), 256, 0, s>>>(stage, uw, nu, tw, nt, tw_at);
   return cudaGetLastError();
 }
 
