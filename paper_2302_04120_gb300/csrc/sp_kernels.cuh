@@ -205,9 +205,12 @@ __global__ void __launch_bounds__(256, PREC == 1 ? 3 : 2) k_moments(const SpPara
   const long long n = (long long)j * P.pitch + i;
   const S *src = (const S *)P.src;
   const bool interior = !P.local && (i > 0) && (i < P.nx - 1) && (j > 0) && (j < P.ny - 1);
-  R f[9], g[9];
-  if (FLOW != FLOW_NONE) pull_f<S, R, SYM>(P, src, i, j, interior, f);
-  if (TH != TH_NONE) pull_g<S, R, ThLat<TH>::Q, SYM>(P, src, i, j, interior, g);
+  // only the lattices that the asked fields need: T comes from g, the others from f (with
+  // buoyancy the velocity from both)
+  const bool need_f = mask & ~8u, need_g = (mask & 8u) || P.buoy;
+  R f[9] = {}, g[9] = {};
+  if (FLOW != FLOW_NONE && need_f) pull_f<S, R, SYM>(P, src, i, j, interior, f);
+  if (TH != TH_NONE && need_g) pull_g<S, R, ThLat<TH>::Q, SYM>(P, src, i, j, interior, g);
   Macro<R> m;
   load_sources<S, R>(P, n, m);
   moments<R, FLOW, TH>(P, f, g, m);
