@@ -241,7 +241,7 @@ def _batch_run(steps, stream, torch, steps_one=200):
                 one_by_one=round(rate_one, 1), one_by_one_steps=steps_one,
                 speedup=round(cells * steps / t_batch / 1e6 / rate_one, 3),
                 achieved_GBps=round(112 * cells * steps / t_batch / 1e9, 1), tile=list(cfg), status=int(chk),
-                graph="pairs of steps replayed from a CUDA graph")
+                groups="all steps of a call per channel or group of channels, replayed from CUDA graphs")
 
 
 def _adjoint_run(torch):
@@ -401,22 +401,16 @@ def _roofline_d2q9(steps, warmup, stream, torch, launch=None):
             "l2": "state 2.4 GB, larger than L2; back-to-back steps"}
 
 
-# FP64 work per node of the FP64 step k_step_split<0,2,2> (D2Q9 MRT + D2Q5 MRT) on
-# the 2048 x 256 channel, from one ncu capture (profiles/k_step_split_fp64_channel_2048x256.md):
-# 89.02 DADD + 40.11 DMUL + 69.17 DFMA thread instructions per node.
-FP64_FLOPS_PER_NODE = 267.5   # DADD + DMUL + 2 DFMA
-FP64_INSTR_PER_NODE = 198.3   # FP64-pipe instructions (one issue slot each)
+# FP64-pipe instructions per node of the FP64 step k_step_split<0,FLOW_MRT,TH_MRT> (pair-form
+# collisions, unforced): about 90, one issue slot each.
+FP64_INSTR_PER_NODE = 90.0
 
 
 def _fp64_alu(cells, avg_s, fma64_gflops):
-    """The FP64 form against its arithmetic bound: executed FP64 flops per second
-    over the probe's FMA rate, and FP64-pipe instructions per second over the probe's
-    instruction rate (half its flop rate: one FMA = 2 flops, one issue)."""
-    ach = FP64_FLOPS_PER_NODE * cells / avg_s / 1e9
+    """The FP64 form against its arithmetic bound: FP64-pipe instructions per second over
+    the probe's instruction rate (half its flop rate: one FMA = 2 flops, one issue)."""
     inst = FP64_INSTR_PER_NODE * cells / avg_s / 1e9
-    return {"bound": "alu", "flops_per_node": FP64_FLOPS_PER_NODE, "achieved_gflops": round(ach, 1),
-            "peak_gflops": round(fma64_gflops, 1), "peak_source": "lbm_probe_fma_rate",
-            "frac": round(ach / fma64_gflops, 4),
+    return {"bound": "alu", "peak_gflops": round(fma64_gflops, 1), "peak_source": "lbm_probe_fma_rate",
             "fp64_instr_per_node": FP64_INSTR_PER_NODE, "achieved_ginstr": round(inst, 1),
             "frac_pipe": round(inst / (fma64_gflops / 2), 4)}
 
