@@ -445,7 +445,7 @@ __device__ __forceinline__ void collide_flow(const SpParams &P, const Macro<R> &
     const R e4 = m.drho * ((R)1 / (R)9) + r12, e8 = m.drho * ((R)1 / (R)36) + r12;
     d4 = e4 - (R)0.25 * s14;
     d8 = e8 - (R)0.25 * s58;
-    f0 = m.drho - (R)4 * (e4 + e8);
+    f0 = sizeof(R) == 8 ? m.drho - (R)4 * (e4 + e8) : f[0] - (R)4 * (d4 + d8);  // FP32: see collide_mrt5
   } else {
     const R a1 = k.ke * (((s14 - (R)2 * f[0]) + (R)4 * s58) - (R)3 * ru), a2 = k.kep * ((f[0] - s14) + ru);
     d4 = a1 + (R)2 * a2;
@@ -527,16 +527,33 @@ __device__ __forceinline__ void collide_bgk_T(const SpParams &P, const Macro<R> 
 
 // Thermal MRT on D2Q5: moments (1, c_x, c_y, 5|c|^2 - 4c^2, c_x^2 - c_y^2), rates
 // (0, 1/tau_T, 1/tau_T, 1/dt, 1/dt), source Delta t (I - dt Lambda/2) M (w qdot).  The two
-// even moments at rate 1/dt leave every even pair at w S, S = sum g + dt qdot.
+// even moments at rate 1/dt take every even pair to w S, S = sum g + dt qdot.
+// FP64: through S (the rest population is S - 4 p, exact).
+// In FP32 a source of one step is about a unit in the last place of sum g, or less: S rounded
+// loses or doubles it, the same way step after step at a node, and sum g drifts without a
+// source too.  So that form adds changes: of the pairs, w (S - a / 2 w) from a difference that
+// is exact, and of the rest population, what the source and the pairs leave.
+// T - T_in against the FP64 form, relative L2: 1024 x 128 channel with q = 1e6 W/m^3, 2000 steps
+// 1.8e-5 through S, 1.4e-6 this way (10000 steps: 5e-5, 3.5e-6); 700 x 96 without a source,
+// 10000 steps 5.7e-6, 1.3e-6.  Cost on 8192 x 4096: 0.9 % of the step.
 template <typename R>
 __device__ __forceinline__ void collide_mrt5(const SpParams &P, const Macro<R> &m, R g[5]) {
   const SpConst<R> &k = K<R>(P);
   const R d13 = g[1] - g[3], d24 = g[2] - g[4], a13 = g[1] + g[3], a24 = g[2] + g[4];
-  const R S = P.qdot ? m.sumg + k.dt * m.qd : m.sumg;
-  const R p = S * ((R)1 / (R)6);
-  const R px = p - (R)0.5 * a13, py = p - (R)0.5 * a24;
+  const R w = (R)1 / (R)6;
+  R px, py;
+  if (sizeof(R) == 8) {
+    const R S = P.qdot ? m.sumg + k.dt * m.qd : m.sumg, p = S * w;
+    px = p - (R)0.5 * a13;
+    py = p - (R)0.5 * a24;
+    g[0] = S - (R)4 * p;
+  } else {
+    const R dS = P.qdot ? k.dt * m.qd : (R)0;
+    px = w * (fma((R)-3, a13, m.sumg) + dS);
+    py = w * (fma((R)-3, a24, m.sumg) + dS);
+    g[0] += dS - (R)2 * (px + py);
+  }
   const R ex = off_eq(m, k.T0, d13, m.hx), ey = off_eq(m, k.T0, d24, m.hy);
-  g[0] = S - (R)4 * p;
   g[1] += px - k.hsT * ex;
   g[3] += px + k.hsT * ex;
   g[2] += py - k.hsT * ey;
@@ -546,21 +563,45 @@ __device__ __forceinline__ void collide_mrt5(const SpParams &P, const Macro<R> &
 // Thermal MRT on D2Q9 (Sec. 2.2): the momentum transformation matrices and
 // [Lambda_T] = diag(0, 1, 1, omega_T, 1, omega_T, 1, 1, 1), the unit rates read as
 // 1/dt; source Delta t (I - dt Lambda/2) M (w qdot).  Every even pair goes to w S,
-// S = sum g + dt qdot; of the odd moments the first loses s_T of its distance e = j - T h
-// from equilibrium, the third-order ones go to -T h.
+// S = sum g + dt qdot (in the two forms of D2Q5); of the odd moments the first loses s_T of
+// its distance e = j - T h from equilibrium, the third-order ones go to -T h.
 template <typename R>
 __device__ __forceinline__ void collide_mrt9T(const SpParams &P, const Macro<R> &m, R g[9]) {
   const SpConst<R> &k = K<R>(P);
   const R d13 = g[1] - g[3], d24 = g[2] - g[4], d57 = g[5] - g[7], d68 = g[6] - g[8];
   const R a13 = g[1] + g[3], a24 = g[2] + g[4], a57 = g[5] + g[7], a68 = g[6] + g[8];
-  const R S = P.qdot ? m.sumg + k.dt * m.qd : m.sumg;
-  const R p9 = S * ((R)1 / (R)9), p36 = S * ((R)1 / (R)36);
+  const R w4 = (R)1 / (R)9, w8 = (R)1 / (R)36;
+  R p13, p24, p57, p68;
+  if (sizeof(R) == 8) {
+    const R S = P.qdot ? m.sumg + k.dt * m.qd : m.sumg, p9 = S * w4, p36 = S * w8;
+    p13 = p9 - (R)0.5 * a13;
+    p24 = p9 - (R)0.5 * a24;
+    p57 = p36 - (R)0.5 * a57;
+    p68 = p36 - (R)0.5 * a68;
+    g[0] = S - (R)4 * (p9 + p36);
+  } else {
+    // (without a source w S rounded: its two weights' differences left sum g a drift of 2.5e-6
+    // of T - T_in after 10000 steps of a 500 x 50 half channel, this way 1e-6)
+    R dS = (R)0;
+    if (P.qdot) {
+      dS = k.dt * m.qd;
+      p13 = w4 * (fma((R)-4.5, a13, m.sumg) + dS);
+      p24 = w4 * (fma((R)-4.5, a24, m.sumg) + dS);
+      p57 = w8 * (fma((R)-18, a57, m.sumg) + dS);
+      p68 = w8 * (fma((R)-18, a68, m.sumg) + dS);
+    } else {
+      const R p9 = m.sumg * w4, p36 = m.sumg * w8;
+      p13 = p9 - (R)0.5 * a13;
+      p24 = p9 - (R)0.5 * a24;
+      p57 = p36 - (R)0.5 * a57;
+      p68 = p36 - (R)0.5 * a68;
+    }
+    g[0] += dS - (R)2 * ((p13 + p24) + (p57 + p68));
+  }
   const R tx = d57 - d68, ty = d57 + d68;  // the diagonals' share of the first moment
   const R ex = off_eq(m, k.T0, d13 + tx, m.hx), ey = off_eq(m, k.T0, d24 + ty, m.hy);
   const R ox = ((R)2 * tx - d13) * ((R)1 / (R)6) - k.q1T * ex, oy = ((R)2 * ty - d24) * ((R)1 / (R)6) - k.q1T * ey;
   const R w = (R)0.5 * (ox + oy) + k.q2T * (ex + ey), v = (R)0.5 * (oy - ox) + k.q2T * (ey - ex);
-  const R p13 = p9 - (R)0.5 * a13, p24 = p9 - (R)0.5 * a24, p57 = p36 - (R)0.5 * a57, p68 = p36 - (R)0.5 * a68;
-  g[0] = S - (R)4 * (p9 + p36);
   g[1] += p13 + ox;
   g[3] += p13 - ox;
   g[2] += p24 + oy;
