@@ -6,6 +6,7 @@
 
 #include "lattice.cuh"
 #include "lbm_internal.cuh"
+#include "reciprocal.cuh"
 
 namespace lbmk {
 
@@ -338,22 +339,6 @@ struct Macro {
   R hx, hy, jx, jy;             // lattice-scaled: u / c and rho u / c
   R sumg, qd, dT, T;            // thermal; dT = T - T0
 };
-
-// 1 / x for a normal x: the hardware's approximate reciprocal and the third-order
-// iteration r (1 + e + e^2), e = 1 - x r (second order in FP32, whose seed already has
-// 23 bits).  Two to four instructions instead of the IEEE division's sequence; within
-// one unit in the last place.
-__device__ __forceinline__ float recip(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return fmaf(r, fmaf(-x, r, 1.0f), r);
-}
-__device__ __forceinline__ double recip(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
 
 template <typename S, typename R>
 __device__ __forceinline__ void load_sources(const SpParams &P, long long n, Macro<R> &m) {

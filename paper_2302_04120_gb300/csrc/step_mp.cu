@@ -33,6 +33,7 @@
 #include "compensated.cuh"
 #include "lattice.cuh"
 #include "lbm_mp.cuh"
+#include "reciprocal.cuh"
 
 namespace lbmk {
 
@@ -91,30 +92,6 @@ template <typename S, typename R>
 __device__ __forceinline__ void pull_z_at(const MpParams &P, const S *sn, R z[9]) {
 #pragma unroll
   for (int q = 0; q < 9; q++) z[q] = (R)sn[q * P.plane - (long long)cy9(q) * P.pitch - cx9(q)];
-}
-
-// 1 / x and 1 / sqrt(x) in the working precision.  FP32: the hardware approximations
-// (one unit in the last place).  FP64: from them by third-order iterations in e, e = 1 -
-// x r or 1 - x y^2 (1 / (1 - e) = 1 + e + e^2 .., 1 / sqrt(1 - e) = 1 + e / 2 + 3 e^2 / 8 ..).
-__device__ __forceinline__ float rcp(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ double rcp(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-// 1 / |g| for g2 = |g|^2 > 0, else 0.
-__device__ __forceinline__ float inv_norm(float g2) { return g2 != 0.0f ? rsqrtf(g2) : 0.0f; }
-__device__ __forceinline__ double inv_norm(double g2) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(g2));
-  const double e = fma(-g2 * y, y, 1.0);
-  y = fma(y * e, fma(e, 0.375, 0.5), y);
-  return g2 > 1e-300 ? y : 0.0;  // a smaller |g|^2 has left the normal range
 }
 
 template <typename S, typename R>
