@@ -21,11 +21,10 @@ struct DevSide {
 // conversion is an instruction of the slow FP64 pipe).
 template <typename R>
 struct SpConst {
-  R c, cs2, dt, rho0, T0, Fx, Fy, ux_pres, uy_pres;
-  R inv_c, inv_cs2, three_inv_c2;  // 1/c, 1/cs2, 3/(c c), each rounded once in R
+  R c, dt, rho0, T0, Fx, Fy, ux_pres, uy_pres;
+  R inv_c, inv_cs2;                 // 1/c, 1/cs2, each rounded once in R
   R hdt;                            // dt / 2
-  R fk_e, fk_eps, fk_q, fk_nu;      // MRT forcing factors (1 - s_k / 2) dt, s_k = dt Lambda_k
-  R omega, s_e, s_eps, s_q, s_nu, omegaT, tsrc_fac, flux_coef, bgx, bgy, T_ref;
+  R omegaT, tsrc_fac, flux_coef, bgx, bgy, T_ref;
   // folded factors of the pair-form collisions (sp_device.cuh), formed in FP64:
   R hdt_ic;                         // dt / (2 c)
   R kq, kn, ke, kep;                // s_q / 6, s_nu / 4, s_e / 36, s_eps / 12
