@@ -670,9 +670,15 @@ static cudaError_t sink_refresh(const lbm_t h, int from, int pre, cudaStream_t s
 //  * above that blocks of two warps in FP32 (2048 x 256: 9.2 with 64 x 4, 6.8 with 64 x 1,
 //    9.5 with 32 x 1, whose 32 blocks per SM leave registers unused) and of four in FP64
 //    (1024 x 128: 30.1, 26.7);
-//  * FP32 with a D2Q5 thermal lattice whose two state buffers exceed the 129 MB L2: the
-//    build for 6 resident blocks per SM with 256 x 1 blocks (8192 x 4096: 545 against 555
-//    with 64 x 1 and 580 with 64 x 4; on the D2Q9 lattice it is slower: 727 against 704).
+//  * FP32 with both lattices on D2Q9 + D2Q5 and more than 200 MB in the two state buffers: the
+//    build for 6 resident blocks per SM with 256 x 1 blocks (8192 x 4096: 545 against 555 with
+//    64 x 1 and 580 with 64 x 4; 260 MB, 2048 to 4096 columns: equal to 64 x 1; 160 MB: 2 to 9 %
+//    slower; on the D2Q9 thermal lattice it is slower: 727 against 704);
+//  * FP32 above 200 MB on grids narrower than a wide block can use (64 columns, 128 where the
+//    build above does not run): the nominal 64 x 4, whose blocks reach over several rows (D2Q9
+//    + D2Q5, 400 MB: 48 columns 143.9 against 155.0 with 256 x 1 and 154.2 with 32 x 2, 33 columns
+//    120.2, 126.4, 125.9, 65 columns 107.0, 106.5, 108.7; D2Q9 + D2Q9 400 MB: 48 columns 138.6,
+//    32 x 2 151.5, 100 columns 89.4, 89.8, 130 columns 88.3, 86.2; 160 MB, 33 columns: 34.2, 31.3).
 // Wide shapes only where the last block of a row wastes little; the shape reported by
 // lbm_launch_config stays the nominal one.
 struct StepLaunch {
@@ -684,12 +690,15 @@ static StepLaunch step_launch(const lbm_t h) {
   StepLaunch l = {h->launch_kind == LBM_LAUNCH_GRID_OCC, h->block};
   if (h->launch_set || h->launch_kind == LBM_LAUNCH_TMA) return l;
   const long long nodes = (long long)h->p.nx * h->p.ny;
-  const int fp64 = h->p.precision == LBM_FP64;
+  const int fp64 = h->p.precision == LBM_FP64, d2q9_d2q5 = h->p.flow && h->p.thermal == LBM_D2Q5;
+  const bool large = !fp64 && 2.0 * h->nq * h->plane * h->elem > 200e6;
   dim3 b;
   int occ = 0;
   if (nodes <= 32ll * h->nsm * (fp64 ? 24 : 32)) {
     b = dim3(32, 1);
-  } else if (!fp64 && h->p.thermal == LBM_D2Q5 && h->p.flow && 2.0 * h->nq * h->plane * h->elem > 129e6) {
+  } else if (large && h->p.nx <= (d2q9_d2q5 ? 64 : 128)) {
+    return l;
+  } else if (large && d2q9_d2q5) {
     b = dim3(256, 1);
     occ = 1;
   } else {
