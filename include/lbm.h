@@ -275,9 +275,10 @@ lbm_status lbm_probe_fma_rate(int precision, double *gflops);
 /*
  * Launch configuration of the single-phase step (no counterpart in the paper: a
  * choice of memory pipeline for the same arithmetic).  cfg[4]:
+ *  {LBM_LAUNCH_AUTO, 0, 0, 0}: a grid launch whose block shape and build the library
+ *     takes by grid size and precision (the default);
  *  {LBM_LAUNCH_GRID, block_x, block_y, 0}: one thread per node, block_x a multiple
- *     of 32, block_x * block_y <= 256 (the default, 64 x 4: until a launch is set here
- *     or by lbm_autotune, the library takes the block shape and the build by grid size);
+ *     of 32, block_x * block_y <= 256;
  *  {LBM_LAUNCH_GRID_OCC, block_x, block_y, 0}: the same kernel built for more
  *     resident blocks per SM (FP32 with a thermal lattice: 6 blocks of 256 threads at
  *     40 registers instead of 4 at 64; faster on large grids, slower on short
@@ -288,13 +289,17 @@ lbm_status lbm_probe_fma_rate(int precision, double *gflops);
  *     `stages` tiles ahead (the first step after lbm_init_fields always uses the
  *     grid launch).  A wait for a box that runs out (about 1 s) marks the handle;
  *     the next lbm_integrals / lbm_check then fails with LBM_ERR_TIMEOUT.
- * lbm_autotune chooses among all three kinds; lbm_launch_config reads the current one.
+ * lbm_autotune chooses among the last three kinds and sets its choice.  lbm_launch_config
+ * reads the launch that is set; while none is, or after LBM_LAUNCH_AUTO, it gives the nominal
+ * {LBM_LAUNCH_GRID, 64, 4, 0}.  Setting that fixes 64 x 4 blocks: a program that puts a
+ * default launch back sets LBM_LAUNCH_AUTO.
  * Errors: LBM_ERR_ARG (two-phase handle, out-of-range value, more CTAs per SM than
  * fit), LBM_ERR_CUDA (the driver refused the tensor maps).
  */
 #define LBM_LAUNCH_GRID 0
 #define LBM_LAUNCH_TMA 1
 #define LBM_LAUNCH_GRID_OCC 2
+#define LBM_LAUNCH_AUTO 3
 lbm_status lbm_set_launch(lbm_t h, const int cfg[4]);
 lbm_status lbm_launch_config(lbm_t h, int cfg[4]);
 

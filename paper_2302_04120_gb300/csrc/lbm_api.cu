@@ -83,6 +83,7 @@ struct StepKey {
   lbmk::MpParams mp[2];
   SpParams sp[2];
 };
+static const dim3 kNominalBlock(64, 4);  // of a grid launch while none is set (see step_launch)
 static constexpr long kGraphSteps = 64;  // even: the ping-pong buffers end where they start
 
 static char g_create_err[512];
@@ -358,7 +359,7 @@ extern "C" lbm_status lbm_create(const lbm_params *pin, void *stream, lbm_t *out
   h->plane = (long long)h->pitch * p.ny;
   if (p.phase) h->nq = 9 + 5 + 2;   // z, h, (phi u)_prev
   else h->nq = (p.flow ? 9 : 0) + (p.thermal ? p.thermal : 0);
-  h->block = dim3(64, 4);
+  h->block = kNominalBlock;
   for (int s = 0; s < 4; s++) {
     h->bc[s] = LBM_BC_PERIODIC;
     h->tbc[s] = LBM_TBC_NONE;
@@ -1524,6 +1525,10 @@ static lbm_status ensure_tmaps(lbm_t h, int ty) {
 
 static lbm_status check_launch(lbm_t h, const int cfg[4]) {
   if (two_phase(h)) return fail(h, LBM_ERR_ARG, "two-phase solves use a fixed 32 x 8 tile");
+  if (cfg[0] == LBM_LAUNCH_AUTO) {
+    if (cfg[1] || cfg[2] || cfg[3]) return fail(h, LBM_ERR_ARG, "automatic launch: the other values must be 0");
+    return LBM_OK;
+  }
   if (cfg[0] == LBM_LAUNCH_GRID || cfg[0] == LBM_LAUNCH_GRID_OCC) {
     if (cfg[1] < 32 || cfg[1] % 32 != 0 || cfg[2] < 1 || cfg[1] * cfg[2] > 256)
       return fail(h, LBM_ERR_ARG, "grid launch: block_x a multiple of 32, block_x * block_y <= 256");
@@ -1539,13 +1544,15 @@ static lbm_status check_launch(lbm_t h, const int cfg[4]) {
       return fail(h, LBM_ERR_ARG, "TMA launch: 1..%d CTAs per SM fit for this tile and stage count", occ);
     return ensure_tmaps(h, cfg[1]);
   }
-  return fail(h, LBM_ERR_ARG, "launch kind must be LBM_LAUNCH_GRID, LBM_LAUNCH_GRID_OCC or LBM_LAUNCH_TMA");
+  return fail(h, LBM_ERR_ARG, "launch kind must be LBM_LAUNCH_GRID, LBM_LAUNCH_GRID_OCC, LBM_LAUNCH_TMA or LBM_LAUNCH_AUTO");
 }
 
 static void apply_launch(lbm_t h, const int cfg[4]) {
-  h->launch_kind = cfg[0];
-  h->launch_set = 1;
-  if (cfg[0] != LBM_LAUNCH_TMA) {
+  h->launch_set = cfg[0] != LBM_LAUNCH_AUTO;
+  h->launch_kind = h->launch_set ? cfg[0] : LBM_LAUNCH_GRID;
+  if (!h->launch_set) {
+    h->block = kNominalBlock;
+  } else if (cfg[0] != LBM_LAUNCH_TMA) {
     h->block = dim3(cfg[1], cfg[2]);
   } else {
     h->tma_ty = cfg[1];
