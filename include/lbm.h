@@ -363,8 +363,10 @@ void lbm_destroy(lbm_t h);
 /*
  * Batched solves: many independent single-phase channels of uneven size advanced
  * together, one kernel launch per time step over a flattened (channel, tile) list,
- * replayed from a CUDA graph; in FP32, where a call takes several steps, group by group
- * (as many channels as stay in L2, each group all the call's steps).  Each channel is an
+ * replayed from a CUDA graph.  In calls of four steps or more, FP32 channels of a size that
+ * runs faster so take all the call's steps as a single solve (with the launch that
+ * lbm_set_launch or the size gives it), one after the other, and the rest share the launches;
+ * which ones depends on the sizes and on the number of steps.  Each channel is an
  * ordinary lbm_t owned by the batch: set its boundaries, sources and initial fields and
  * read its moments with the calls above (lbm_batch_channel), but advance it only with
  * lbm_batch_step.
@@ -373,13 +375,19 @@ void lbm_destroy(lbm_t h);
  *                    cannot use the legacy default stream).  Errors as lbm_create.
  *  lbm_batch_step    advance every channel n steps; all channels must be initialised and
  *                    in step.  Asynchronous on the batch stream.  Errors: LBM_ERR_STATE,
- *                    LBM_ERR_ARG (a channel with a lagged sink), LBM_ERR_CUDA.
+ *                    LBM_ERR_ARG (a channel with a lagged sink), LBM_ERR_CUDA (channels
+ *                    may then be at different steps: later calls are refused until every
+ *                    channel has been initialised again).
  *  lbm_batch_autotune time candidate tile shapes (32..256 threads) and grid sizes (1..16
- *                    blocks per SM) on the next step without advancing the solution; keeps
- *                    the fastest; out_cfg (may be NULL) receives {tile_x, tile_y, grid}.
- *  lbm_batch_config  set tile shape and grid explicitly (tile_x * tile_y a multiple of 32,
- *                    at most 256).
- * Every channel's result equals stepping it alone with lbm_step (same arithmetic).
+ *                    blocks per SM) on the next step, as one launch over all channels,
+ *                    without advancing the solution; keeps the fastest; out_cfg (may be
+ *                    NULL) receives {tile_x, tile_y, grid}.  They apply to the shared
+ *                    launches, not to channels that run as single solves.
+ *  lbm_batch_config  set tile shape and grid of the shared launches explicitly (tile_x *
+ *                    tile_y a multiple of 32, at most 256).
+ * Every channel's result equals stepping it alone with lbm_step (same arithmetic; the
+ * kernels compile it in different places, so that in the last places FP32 results depend on
+ * whether a channel shared the launches).
  */
 typedef struct lbm_batch_s *lbm_batch_t;
 lbm_status lbm_batch_create(const lbm_params *params, int n, void *stream, lbm_batch_t *out);

@@ -982,13 +982,16 @@ struct lbm_batch_s {
   // device tables: parity p, channel k at [p * n + k]; local variant at [2n + k]
   SpParams *h_tab, *d_tab;
   int tab_valid;
-  // tile list for the chosen tile shape
+  // tile lists for the chosen tile shape: 0 every channel, 1 + c those that share the launches
+  // of a call of class c; list l is d_tiles[tile0[l]] .. d_tiles[tile0[l + 1] - 1]
   int4 *d_tiles;
-  int ntiles, tiles_bx, tiles_by;
+  int tile0[4], tiles_bx, tiles_by;
   int bx, by, grid;       // launch configuration (autotuned or set)
-  int *order, *first;     // channels group by group; group g is order[first[g]] .. order[first[g + 1] - 1]
-  int *tile0;             // its entries are tiles tile0[g] .. tile0[g + 1] - 1
-  int ngroups;
+  // calls of fewer (c = 0) and of at least kGraphSteps (c = 1) steps: alone[c * n + k], channel
+  // k takes its steps as a single solve; how many do
+  unsigned char *alone;
+  int nalone[2];
+  int torn;               // a call failed after some channels had taken its steps
   cudaGraph_t graph;
   cudaGraphExec_t exec;   // two steps: parity 0 then parity 1
   char err[512];
@@ -1025,53 +1028,62 @@ extern "C" void lbm_batch_destroy(lbm_batch_t b) {
   for (int k = 0; k < b->n; k++) lbm_destroy(b->ch[k]);
   free(b->ch);
   free(b->h_tab);
-  free(b->order);
-  free(b->first);
-  free(b->tile0);
+  free(b->alone);
   cudaFree(b->d_tab);
   cudaFree(b->d_tiles);
   if (b->own_stream) cudaStreamDestroy(b->stream);
   free(b);
 }
 
-// How a batch of FP32 channels is split (kGroupMinSteps: fewer steps of one call reuse too
-// little).  Measured on GB300, MRT + D2Q5 MRT channels, billions of node updates per second,
-// back-to-back steps of one channel of n thousand nodes (state_bytes MB) as a single solve and
-// as one batched launch per step:
-//   66 (7 MB): 17 and 6;  131 (15 MB): 30 and 11;  262 (29 MB): 51 and 20;  524 (59 MB): 75
-//   and 32;  768 (86 MB): 76 and 39;  1024 (115 MB): 60 and 42;  3200 (358 MB): 59 and 49.
-// So a channel of more than 16 MB runs as a single solve (parameters in constant memory, the
-// frame spread over the SMs); smaller ones share launches, as many as fill 60 MB (48 uneven
-// channels, 48 steps: 25.4 ms with 60 MB, 25.7 with 80, 26.1 with 40 or 110, 26.7 with one
-// launch per step over all, in a first form that took single solves from half of that size).
-constexpr double kAloneBytes = 16e6, kGroupBytes = 60e6;
-constexpr long kGroupMinSteps = 4;
+// Which FP32 channels take a call's steps as a single solve, one after the other, while the
+// others share one launch per step.  A single solve runs all the steps before the next channel's
+// turn, so that a state below the 129 MB L2 stays there, and its frame is spread over the
+// SMs; but a step of it fills the chip only from some size on.  Measured on GB300, MRT + D2Q5
+// MRT, billions of node updates per second, 16 equal channels of the given size (both buffers),
+// one launch over all against single solves:
+//   calls of 48 steps (4 and 8: the same order): 20 MB 41 and 23, 30 MB 43 and 33, 42 MB 45 and
+//   45, 50 MB 47 and 54, 60 MB 48 and 56, 80 MB 49 and 60, 100 MB 50 and 54, 120 MB 48 and 52,
+//   140 MB 51 and 47, 180 MB 50 and 48, 300 MB 49 and 55 (by then with the build for large grids);
+//   calls of 200 steps, which replay graphs (host calls hidden): 25 MB 45 and 42, 35 MB 46 and
+//   54, 42 MB 46 and 63, 60 MB 50 and 75, 100 MB 50 and 65, 140 MB 51 and 52, 180 MB 50 and 52,
+//   300 MB 49 and 58.
+// Sharing launches in groups that stay in L2 lost against one launch over all (48 channels of
+// 5 MB: 37 over all, 27 in groups of 60 MB, 34 of 90 MB; of 16 MB: 42, 26, 36).  The launches of
+// the others cost a few us per step that their nodes would not cost in the launch over all,
+// so single solves have to be worth them (one of 60 MB beside four of 1 MB: 17.4 us a step over
+// all, 17.8 split; four of 60 MB: 49.1 and 46.4).
+constexpr long kAloneMinSteps = 4;
+constexpr double kAloneTotal = 200e6;
 
 static double state_bytes(const lbm_t h) { return 2.0 * h->nq * h->plane * h->elem; }
-static bool batch_alone(const lbm_t h) { return state_bytes(h) > kAloneBytes; }
+static bool batch_alone(const lbm_t h, int c) {
+  if (h->p.precision == LBM_FP64 || h->launch_kind == LBM_LAUNCH_TMA) return false;
+  const dim3 blk = step_launch(h).block;  // (a shape set by the caller may need too many rows of blocks)
+  if ((h->p.ny + blk.y - 1) / blk.y > 65535) return false;
+  const double s = state_bytes(h);
+  return c ? s > 32e6 : (s > 55e6 && s < 129e6) || s > 240e6;
+}
 
-// Groups: every channel alone that can be, the others in order of index
-// as long as their state fits.
-static void batch_groups(lbm_batch_t b) {
-  int at = 0;
-  b->ngroups = 0;
-  for (int k = 0; k < b->n; k++)
-    if (batch_alone(b->ch[k])) {
-      b->first[b->ngroups++] = at;
-      b->order[at++] = k;
+// Brings alone[] up to date with the channels' launches; whether it changed.
+static bool batch_split(lbm_batch_t b) {
+  bool changed = false;
+  for (int c = 0; c < 2; c++) {
+    int count = 0;
+    double bytes = 0.0;
+    for (int k = 0; k < b->n; k++)
+      if (batch_alone(b->ch[k], c)) {
+        count++;
+        bytes += state_bytes(b->ch[k]);
+      }
+    if (count < b->n && bytes < kAloneTotal) count = 0;
+    for (int k = 0; k < b->n; k++) {
+      const unsigned char a = count && batch_alone(b->ch[k], c);
+      changed = changed || b->alone[c * b->n + k] != a;
+      b->alone[c * b->n + k] = a;
     }
-  double held = 2.0 * kGroupBytes;
-  for (int k = 0; k < b->n; k++) {
-    if (batch_alone(b->ch[k])) continue;
-    const double need = state_bytes(b->ch[k]);
-    if (held + need > kGroupBytes) {
-      b->first[b->ngroups++] = at;
-      held = 0.0;
-    }
-    held += need;
-    b->order[at++] = k;
+    b->nalone[c] = count;
   }
-  b->first[b->ngroups] = at;
+  return changed;
 }
 
 extern "C" lbm_status lbm_batch_create(const lbm_params *params, int n, void *stream, lbm_batch_t *out) {
@@ -1090,10 +1102,8 @@ extern "C" lbm_status lbm_batch_create(const lbm_params *params, int n, void *st
   b->n = n;
   b->ch = (lbm_t *)calloc(n, sizeof(lbm_t));
   b->h_tab = (SpParams *)calloc(3 * (size_t)n, sizeof(SpParams));
-  b->order = (int *)malloc(n * sizeof(int));
-  b->first = (int *)malloc((n + 1) * sizeof(int));
-  b->tile0 = (int *)malloc((n + 1) * sizeof(int));
-  if (!b->ch || !b->h_tab || !b->order || !b->first || !b->tile0) {
+  b->alone = (unsigned char *)calloc(2 * (size_t)n, 1);
+  if (!b->ch || !b->h_tab || !b->alone) {
     b->n = b->ch ? n : 0;
     lbm_batch_destroy(b);
     return bfail(NULL, LBM_ERR_NOMEM, "host allocation failed");
@@ -1116,7 +1126,7 @@ extern "C" lbm_status lbm_batch_create(const lbm_params *params, int n, void *st
       return bfail(NULL, st, "%s", msg);
     }
   }
-  batch_groups(b);
+  batch_split(b);
   b->prec = params[0].precision;
   sp_kinds(b->ch[0], &b->flow, &b->th);
   if (cudaMalloc(&b->d_tab, 3 * (size_t)n * sizeof(SpParams)) != cudaSuccess) {
@@ -1141,35 +1151,38 @@ extern "C" lbm_t lbm_batch_channel(lbm_batch_t b, int k) {
 
 extern "C" int lbm_batch_size(lbm_batch_t b) { return b ? b->n : 0; }
 
-// (Re)build the entry list for a tile shape: group by group, every channel's boundary
-// frame in chunks of bx*by nodes first (the longest-running nodes start first), then the
-// interior tiles.
-static lbm_status batch_tiles(lbm_batch_t b, int bx, int by) {
-  if (b->d_tiles && b->tiles_bx == bx && b->tiles_by == by) return LBM_OK;
+// (Re)build the entry lists for a tile shape (rebuild: also where it is the same): of every
+// list the boundary frames in chunks of bx*by nodes first (the longest-running nodes start
+// first), then the interior tiles.
+static lbm_status batch_tiles(lbm_batch_t b, int bx, int by, bool rebuild) {
+  if (b->d_tiles && b->tiles_bx == bx && b->tiles_by == by && !rebuild) return LBM_OK;
   const int chunk = bx * by;
+  auto listed = [&](int l, int k) { return l == 0 || !b->alone[(l - 1) * b->n + k]; };
   long long total = 0;
-  for (int k = 0; k < b->n; k++) {
-    const int nx = b->ch[k]->p.nx, ny = b->ch[k]->p.ny;
-    total += (lbmk::frame_nodes(nx, ny) + chunk - 1) / chunk;
-    total += (long long)((nx + bx - 1) / bx) * ((ny + by - 1) / by);
-  }
+  for (int l = 0; l < 3; l++)
+    for (int k = 0; k < b->n; k++) {
+      if (!listed(l, k)) continue;
+      const int nx = b->ch[k]->p.nx, ny = b->ch[k]->p.ny;
+      total += (lbmk::frame_nodes(nx, ny) + chunk - 1) / chunk;
+      total += (long long)((nx + bx - 1) / bx) * ((ny + by - 1) / by);
+    }
   if (total > (1ll << 31) - 1) return bfail(b, LBM_ERR_ARG, "too many tiles");
   int4 *h = (int4 *)malloc(sizeof(int4) * (size_t)total);
   if (!h) return bfail(b, LBM_ERR_NOMEM, "host allocation failed");
   long long t = 0;
-  for (int g = 0; g < b->ngroups; g++) {
-    b->tile0[g] = (int)t;
-    for (int o = b->first[g]; o < b->first[g + 1]; o++) {
-      const int k = b->order[o], nf = lbmk::frame_nodes(b->ch[k]->p.nx, b->ch[k]->p.ny);
-      for (int f0 = 0; f0 < nf; f0 += chunk) h[t++] = make_int4(k, f0, 0, 1);
+  for (int l = 0; l < 3; l++) {
+    b->tile0[l] = (int)t;
+    for (int k = 0; k < b->n; k++) {
+      const int nf = lbmk::frame_nodes(b->ch[k]->p.nx, b->ch[k]->p.ny);
+      for (int f0 = 0; listed(l, k) && f0 < nf; f0 += chunk) h[t++] = make_int4(k, f0, 0, 1);
     }
-    for (int o = b->first[g]; o < b->first[g + 1]; o++) {
-      const int k = b->order[o], nx = b->ch[k]->p.nx, ny = b->ch[k]->p.ny;
-      for (int y0 = 0; y0 < ny; y0 += by)
+    for (int k = 0; k < b->n; k++) {
+      const int nx = b->ch[k]->p.nx, ny = b->ch[k]->p.ny;
+      for (int y0 = 0; listed(l, k) && y0 < ny; y0 += by)
         for (int x0 = 0; x0 < nx; x0 += bx) h[t++] = make_int4(k, x0, y0, 0);
     }
   }
-  b->tile0[b->ngroups] = (int)t;
+  b->tile0[3] = (int)t;
   cudaStreamSynchronize(b->stream);
   cudaFree(b->d_tiles);
   b->d_tiles = NULL;
@@ -1177,7 +1190,6 @@ static lbm_status batch_tiles(lbm_batch_t b, int bx, int by) {
   if (e == cudaSuccess) e = cudaMemcpy(b->d_tiles, h, sizeof(int4) * (size_t)total, cudaMemcpyHostToDevice);
   free(h);
   if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, "tile list: %s", cudaGetErrorString(e));
-  b->ntiles = (int)total;
   b->tiles_bx = bx;
   b->tiles_by = by;
   batch_drop_graph(b);
@@ -1192,7 +1204,10 @@ static lbm_status batch_tables(lbm_batch_t b, int *cur, int *pre) {
     if (!h->initialised) return bfail(b, LBM_ERR_STATE, "channel %d is not initialised", k);
     if (h->cur != c0 || h->pre != p0)
       return bfail(b, LBM_ERR_STATE, "channel %d is not in step with channel 0 (step it through the batch only)", k);
+    if (b->torn && h->steps != b->ch[0]->steps)
+      return bfail(b, LBM_ERR_STATE, "an earlier call failed part-way: initialise every channel again (channel %d)", k);
   }
+  b->torn = 0;
   SpParams *tmp = (SpParams *)malloc(3 * (size_t)b->n * sizeof(SpParams));
   if (!tmp) return bfail(b, LBM_ERR_NOMEM, "host allocation failed");
   for (int k = 0; k < b->n; k++) {
@@ -1219,9 +1234,11 @@ static lbm_status batch_tables(lbm_batch_t b, int *cur, int *pre) {
   return LBM_OK;
 }
 
-static cudaError_t batch_launch(lbm_batch_t b, const SpParams *table) {
-  return lbmk::sp_batch_step(table, b->d_tiles, b->ntiles, b->prec, b->flow, b->th, dim3(b->bx, b->by), b->grid,
-                             b->stream);
+// One launch over the tiles of list l (0: every channel).
+static cudaError_t batch_launch(lbm_batch_t b, const SpParams *table, int l = 0) {
+  const int nt = b->tile0[l + 1] - b->tile0[l];
+  return lbmk::sp_batch_step(table, b->d_tiles + b->tile0[l], nt, b->prec, b->flow, b->th, dim3(b->bx, b->by),
+                             l && b->grid > nt ? nt : b->grid, b->stream);
 }
 
 static void batch_advance(lbm_batch_t b, long n) {
@@ -1237,7 +1254,7 @@ extern "C" lbm_status lbm_batch_config(lbm_batch_t b, int bx, int by, int grid) 
   if (!b) return bfail(b, LBM_ERR_ARG, "NULL batch");
   if (bx < 1 || by < 1 || bx * by > 256 || (bx * by) % 32 || grid < 1)
     return bfail(b, LBM_ERR_ARG, "tile must be a multiple of 32 threads, at most 256; grid >= 1");
-  lbm_status st = batch_tiles(b, bx, by);
+  lbm_status st = batch_tiles(b, bx, by, false);
   if (st != LBM_OK) return st;
   if (b->bx != bx || b->by != by || b->grid != grid) batch_drop_graph(b);
   b->bx = bx;
@@ -1252,7 +1269,8 @@ extern "C" lbm_status lbm_batch_step(lbm_batch_t b, long n) {
   if (n == 0) return LBM_OK;
   for (int k = 0; k < b->n; k++)  // the batched launch does not refresh a lagged qdot
     if (b->ch[k]->sink_conv != 0.0) return bfail(b, LBM_ERR_ARG, "channel %d has a lagged sink", k);
-  lbm_status st = batch_tiles(b, b->bx, b->by);
+  const bool changed = batch_split(b);
+  lbm_status st = batch_tiles(b, b->bx, b->by, changed);
   if (st != LBM_OK) return st;
   int cur, pre;
   st = batch_tables(b, &cur, &pre);
@@ -1263,27 +1281,22 @@ extern "C" lbm_status lbm_batch_step(lbm_batch_t b, long n) {
     n--;
     cur = 1 - cur;
   }
-  // FP32: each group takes all n steps before the next one, so that its state stays in L2
-  // (one launch per step over all channels streams every state from HBM each step).  FP64
-  // steps are bound by the FP64 pipe and keep one launch per step.
-  if (b->prec != LBM_FP64 && (b->ngroups > 1 || batch_alone(b->ch[0])) && n >= kGroupMinSteps) {
-    for (int g = 0; g < b->ngroups; g++) {
-      lbm_t h = b->ch[b->order[b->first[g]]];
-      if (batch_alone(h) && h->launch_kind != LBM_LAUNCH_TMA) {
-        st = advance(h, n);
-        if (st != LBM_OK) return bfail(b, st, "channel %d: %s", b->order[b->first[g]], h->err);
-        continue;
-      }
-      const int nt = b->tile0[g + 1] - b->tile0[g];
-      for (long s = 0; s < n; s++)
-        BCU(b, lbmk::sp_batch_step(b->d_tab + (size_t)((cur + s) & 1) * b->n, b->d_tiles + b->tile0[g], nt, b->prec, b->flow,
-                                   b->th, dim3(b->bx, b->by), b->grid < nt ? b->grid : nt, b->stream));
-      for (int o = b->first[g]; o < b->first[g + 1]; o++) {
-        lbm_t c = b->ch[b->order[o]];
-        c->cur = (int)((c->cur + n) & 1);
-        c->steps += n;
-      }
+  const int c = n >= kGraphSteps;
+  if (n >= kAloneMinSteps && b->nalone[c]) {  // (FP32)
+    b->torn = 1;  // until every channel has taken the steps
+    for (int k = 0; k < b->n; k++) {
+      if (!b->alone[c * b->n + k]) continue;
+      st = advance(b->ch[k], n);
+      if (st != LBM_OK) return bfail(b, st, "channel %d: %s", k, b->ch[k]->err);
     }
+    if (b->nalone[c] < b->n)
+      for (long s = 0; s < n; s++) BCU(b, batch_launch(b, b->d_tab + (size_t)((cur + s) & 1) * b->n, 1 + c));
+    for (int k = 0; k < b->n; k++) {
+      if (b->alone[c * b->n + k]) continue;
+      b->ch[k]->cur = (int)((b->ch[k]->cur + n) & 1);
+      b->ch[k]->steps += n;
+    }
+    b->torn = 0;
     return LBM_OK;
   }
   if (n > 0 && cur == 1) {  // align to parity 0 for the two-step graph
@@ -1333,7 +1346,7 @@ extern "C" lbm_status lbm_batch_autotune(lbm_batch_t b, int out_cfg[3]) {
   float best = 1e30f;
   int bb[3] = {b->bx, b->by, b->grid};
   for (const auto &sh : shapes) {
-    st = batch_tiles(b, sh[0], sh[1]);
+    st = batch_tiles(b, sh[0], sh[1], false);
     if (st != LBM_OK) break;
     const int occ = lbmk::sp_batch_occupancy(b->prec, b->flow, b->th, sh[0] * sh[1]);
     // grid-stride launches of a few blocks per SM, and one block per entry (the block
@@ -1341,7 +1354,7 @@ extern "C" lbm_status lbm_batch_autotune(lbm_batch_t b, int out_cfg[3]) {
     for (int mi = 0; mi <= (int)(sizeof(mults) / sizeof(mults[0])); mi++) {
       const int m = mi < (int)(sizeof(mults) / sizeof(mults[0])) ? mults[mi] : 0;
       if (m > (occ > 0 ? occ : 1) * 2) continue;
-      const int grid = m ? sms * m : b->ntiles;
+      const int grid = m ? sms * m : b->tile0[1];
       b->bx = sh[0];
       b->by = sh[1];
       b->grid = grid;
