@@ -166,11 +166,10 @@ __global__ void k_adj_loss(const SpParams P, const double *Ttarget, R *LP, doubl
 
 // The node's share of a reverse step after Lam_X(t) is known: pre(t) from X_{t-1}, the
 // transposed collisions (the pair forms of sp_device.cuh, reversed line by line), the
-// parameter gradients and Lam_pre(t).  Returns this node's share of dL/dnu (cn, cq: ds_nu
-// / dnu and ds_q / dnu).
+// parameter gradients and Lam_pre(t).  dn, dq: this node's share of 4 dL/ds_nu and 6 dL/ds_q.
 template <typename S, typename R, bool INNER>
-__device__ __forceinline__ R reverse_node(const SpParams &P, int i, int j, R lx[9], R lg[5], R *LP, double *grad_qdot,
-                                          R cn, R cq) {
+__device__ __forceinline__ void reverse_node(const SpParams &P, int i, int j, R lx[9], R lg[5], R *LP, double *grad_qdot,
+                                             R &dn, R &dq) {
   const long long n = nidx(P, i, j);
   const SpConst<R> &k = K<R>(P);
   const S *src = (const S *)P.src;
@@ -235,12 +234,12 @@ __device__ __forceinline__ R reverse_node(const SpParams &P, int i, int j, R lx[
   const R u2 = two * (lru + bX), v2 = two * (lru - bX);
   R Jx = u2 * hx + bY * hy, Jy = v2 * hy + bY * hx;
   lr -= half * (hx * Jx + hy * Jy);
-  // d L / d s_nu and d L / d s_q
+  // 4 d L / d s_nu and 6 d L / d s_q
   const R xx = (f[1] + f[3]) - (f[2] + f[4]), xy = (f[5] + f[7]) - (f[6] + f[8]);
   const R tx = (f[5] - f[7]) - (f[6] - f[8]), ty = (f[5] - f[7]) + (f[6] - f[8]);
   const R xx0 = m.jx * hx;
-  R dn = AX * ((xx0 - m.jy * hy) - xx) + AY * (m.jx * hy - xy);
-  R dq = Ox * ((tx + m.jx) - two * (f[1] - f[3])) + Oy * ((ty + m.jy) - two * (f[2] - f[4]));
+  dn = AX * ((xx0 - m.jy * hy) - xx) + AY * (m.jx * hy - xy);
+  dq = Ox * ((tx + m.jx) - two * (f[1] - f[3])) + Oy * ((ty + m.jy) - two * (f[2] - f[4]));
   if (P.forced) {
     const R px = m.Fx * k.inv_c, py = m.Fy * k.inv_c;
     const R gX = k.gn * AX, gY = half * k.gn * AY;
@@ -270,7 +269,6 @@ __device__ __forceinline__ R reverse_node(const SpParams &P, int i, int j, R lx[
   LP[7 * P.plane + n] = a57 - d57;
   LP[6 * P.plane + n] = a68 + d68;
   LP[8 * P.plane + n] = a68 - d68;
-  return cn * ((R)0.25 * dn) + cq * (dq * ((R)1 / (R)6));
 }
 
 // Nodes within two cells of a side, each once: the rows j < 2 and j >= ny - 2, then the
@@ -302,22 +300,23 @@ __device__ __forceinline__ bool adj_frame_node(int nx, int ny, int f, int &i, in
 // consumers are all ordinary streaming links, with the boundary code compiled out: in one
 // mixed launch the step waited for the warps that ran both paths one after the other and
 // for their code.
+// cn, cq: (1/4) d s_nu / d nu and (1/6) d s_q / d nu.
 // Blocks of two warps: nothing is shared between warps (each adds its own dL/dnu partial,
-// one compensated sum in a fixed order), so no warp waits at a barrier.
+// summed in a fixed order), so no warp waits at a barrier.
 // Measured on 1024 x 128 (one launch, cold caches): FP64 129 -> 47 us (348 -> about 150 FP64
 // instructions per node), FP32 28 -> 15.7 us.
 constexpr int kAdjThreads = 64;
 template <typename S, typename R>
 __global__ void __launch_bounds__(kAdjThreads, sizeof(R) == 4 ? 16 : 8) k_adj_step(
     const SpParams P, int nfb, int gx, const S *__restrict__ Xt, const R *__restrict__ LPn, R *__restrict__ LP, double *grad_qdot,
-    double *grad_flux2, double *grad_flux3, R cn, R cq, double *nu_partials) {
-  R dnu = 0;
+    double *grad_flux2, double *grad_flux3, double cn, double cq, double *nu_partials) {
+  R dn = 0, dq = 0;
   int i, j;
   R lx[9], lg[5];
   if ((int)blockIdx.x < nfb) {
     if (adj_frame_node(P.nx, P.ny, blockIdx.x * kAdjThreads + threadIdx.x, i, j)) {
       gather_frame<S, R>(P, Xt, LPn, i, j, lx, lg, grad_flux2, grad_flux3);
-      dnu = reverse_node<S, R, false>(P, i, j, lx, lg, LP, grad_qdot, cn, cq);
+      reverse_node<S, R, false>(P, i, j, lx, lg, LP, grad_qdot, dn, dq);
     }
   } else {
     j = (blockIdx.x - nfb) / gx;
@@ -329,15 +328,20 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(R) == 4 ? 16 : 8) k_adj_st
       for (int q = 0; q < 9; q++) lx[q] = LPn[q * P.plane + n + (long long)cy9(q) * P.pitch + cx9(q)];
 #pragma unroll
       for (int q = 0; q < 5; q++) lg[q] = LPng[q * P.plane + n + (long long)cy5(q) * P.pitch + cx5(q)];
-      dnu = reverse_node<S, R, true>(P, i, j, lx, lg, LP, grad_qdot, cn, cq);
+      reverse_node<S, R, true>(P, i, j, lx, lg, LP, grad_qdot, dn, dq);
     }
   }
+  // the lower half of the warp sums dn, the upper half dq, in the working precision; their
+  // factors, which FP32 would round and whose products cancel, come in FP64 once per warp
+  const bool upper = threadIdx.x & 16;
   NodeSum<R> sum;
   sum.clear();
-  sum.add(dnu);
-  sum.warp_reduce();
-  if ((threadIdx.x & 31) == 0)
-    nu_partials[blockIdx.x * (kAdjThreads / 32) + threadIdx.x / 32] += sum.value();
+  sum.add(upper ? dq : dn);
+  sum.add(__shfl_xor_sync(0xffffffffu, upper ? dn : dq, 16));
+  sum.template warp_reduce<16>();
+  double v = (upper ? cq : cn) * sum.value();
+  v += __shfl_down_sync(0xffffffffu, v, 16);
+  if ((threadIdx.x & 31) == 0) nu_partials[blockIdx.x * (kAdjThreads / 32) + threadIdx.x / 32] += v;
 }
 
 __global__ void k_adj_final(const double *nu_partials, long long nb, double *out) {
@@ -381,11 +385,11 @@ cudaError_t adj_step(const SpParams &P, int prec, const void *Xt, const void *LP
   const unsigned nb = adj_blocks(P.nx, P.ny, &nfb, &gx);
   if (prec == 0)
     k_adj_step<double, double><<<nb, kAdjThreads, 0, s>>>(P, nfb, gx, (const double *)Xt, (const double *)LPn,
-                                                          (double *)LP, grad_qdot, grad_flux2, grad_flux3, cn, cq,
-                                                          nu_partials);
+                                                          (double *)LP, grad_qdot, grad_flux2, grad_flux3, 0.25 * cn,
+                                                          cq / 6.0, nu_partials);
   else
     k_adj_step<float, float><<<nb, kAdjThreads, 0, s>>>(P, nfb, gx, (const float *)Xt, (const float *)LPn, (float *)LP,
-                                                        grad_qdot, grad_flux2, grad_flux3, (float)cn, (float)cq,
+                                                        grad_qdot, grad_flux2, grad_flux3, 0.25 * cn, cq / 6.0,
                                                         nu_partials);
   return cudaGetLastError();
 }

@@ -23,9 +23,9 @@ template <> struct NodeSum<double> {
   __device__ void clear() { v = 0.0; }
   __device__ void add(double x) { v += x; }
   __device__ void merge(const NodeSum &o) { v += o.v; }
-  __device__ void warp_reduce() {
+  template <int W = 32> __device__ void warp_reduce() {  // over W lanes: lanes 0, W, .. hold the sums
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    for (int o = W / 2; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   }
   __device__ double value() const { return v; }
 };
@@ -42,9 +42,9 @@ template <> struct NodeSum<float> {
     two_sum(hi, o.hi, hi, e);
     lo += o.lo + e;
   }
-  __device__ void warp_reduce() {
+  template <int W = 32> __device__ void warp_reduce() {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = W / 2; o > 0; o >>= 1) {
       NodeSum x;
       x.hi = __shfl_down_sync(0xffffffffu, hi, o);
       x.lo = __shfl_down_sync(0xffffffffu, lo, o);
