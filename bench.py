@@ -200,8 +200,9 @@ def _e2e(prec, steps, warmup, stream, torch):
 
 def _batch_run(steps, stream, torch, steps_one=200):
     """The batched workload: 256 seeded channels of uneven size (1.5e8 nodes, FP32
-    deviation storage), its `steps` steps in one launch per step with autotuned tiles,
-    against the same channels stepped one by one (one launch per channel per step) over
+    deviation storage), its `steps` steps in one call (channels that run faster so as single
+    solves, the others in one launch per step with autotuned tiles), against the same
+    channels stepped one by one (one launch per channel per step) over
     `steps_one` steps.  The state (16.8 GB) is far larger than L2, so no flush is
     needed."""
     from paper_2302_04120_gb300 import lbm
@@ -241,7 +242,8 @@ def _batch_run(steps, stream, torch, steps_one=200):
                 one_by_one=round(rate_one, 1), one_by_one_steps=steps_one,
                 speedup=round(cells * steps / t_batch / 1e6 / rate_one, 3),
                 achieved_GBps=round(112 * cells * steps / t_batch / 1e9, 1), tile=list(cfg), status=int(chk),
-                groups="all steps of a call per channel or group of channels, replayed from CUDA graphs")
+                groups="channels above 32 MB of state take the call's steps as single solves (CUDA graphs), one after "
+                       "the other; the others share one launch per step, to which tile applies")
 
 
 def _adjoint_run(torch):
@@ -293,8 +295,8 @@ def _adjoint_run(torch):
 
 def _two_phase_run(steps, stream, torch):
     """The bubble workload (512 x 512, saturated water 25 C): per-step time of the
-    one-launch two-phase step with an L2 flush between steps, FP32 (FP64 rho/u/p
-    recovery across the interface) and FP64; plus a 4096 x 4096 roofline-size run."""
+    one-launch two-phase step with an L2 flush between steps, FP32 (rho, u, p recovered
+    in pairs of floats across the interface and in the gas) and FP64; plus a 4096 x 4096 roofline-size run."""
     from paper_2302_04120_gb300 import lbm
     from paper_2302_04120_gb300 import workloads as wl
     flush = torch.empty(512 * 1024 * 1024 // 4, dtype=torch.float32, device="cuda")
@@ -401,9 +403,9 @@ def _roofline_d2q9(steps, warmup, stream, torch, launch=None):
             "l2": "state 2.4 GB, larger than L2; back-to-back steps"}
 
 
-# FP64-pipe instructions per node of the FP64 step k_step_split<0,FLOW_MRT,TH_MRT> (pair-form
-# collisions, unforced): about 90, one issue slot each.
-FP64_INSTR_PER_NODE = 90.0
+# FP64-pipe instructions per node of the FP64 step k_step_split<0,FLOW_MRT,TH_MRT>, unforced: DADD,
+# DMUL and DFMA counted by ncu over one launch (profiles/k_step_split_fp64_channel_2048x256.md).
+FP64_INSTR_PER_NODE = 94.1
 
 
 def _fp64_alu(cells, avg_s, fma64_gflops):
@@ -521,7 +523,8 @@ def run_ours(args):
         return
     if args.profile_batch:
         # only the first 16 channels of the batched workload (1.35e7 nodes, 1.5 GB of
-        # state, above L2), batched, for profiler captures of the batched step kernel
+        # state, above L2), batched, for profiler captures of the batched step kernel: in calls
+        # of one step, which are one launch over all channels
         from paper_2302_04120_gb300 import workloads as wl
         specs = wl.channel_batch_specs()[:16]
         b = lbm.Batch([wl.channel(nx=sp["nx"], ny=sp["ny"], steps=0, Re=sp["Re"], Pr=sp["Pr"], dx=sp["dx"],
@@ -533,11 +536,13 @@ def run_ours(args):
             ch.init(**w["init"])
         b.step(2)
         b.autotune()
-        b.step(args.warmup)
+        for _ in range(args.warmup):
+            b.step(1)
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         torch.cuda.synchronize()
         e0.record(stream)
-        b.step(args.steps)
+        for _ in range(args.steps):
+            b.step(1)
         e1.record(stream)
         torch.cuda.synchronize()
         nodes = sum(sp["nx"] * sp["ny"] for sp in specs)

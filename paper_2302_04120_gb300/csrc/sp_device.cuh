@@ -330,7 +330,7 @@ __device__ __forceinline__ void pull_g(const SpParams &P, const S *src, int i, i
 // Why in this form: on GB300 the FP64 pipe issues one warp instruction every 16 cycles
 // per SM and bounds the FP64 step, so the count of FP64 instructions per node is its
 // time.  The unfolded form (moments, equilibria and forcing of all nine rates, then
-// M^-1) took 198 per node of D2Q9 MRT + D2Q5 MRT, this one about 90.  Measured, back-to-back
+// M^-1) took 198 per node of D2Q9 MRT + D2Q5 MRT, this one 94.  Measured, back-to-back
 // steps: FP64 2048 x 256 191.6 -> 102.4 us, FP64 64 x 33 BGK 14.6 -> 8.5 us, FP32 2048 x 256
 // 10.1 -> 9.1 us; the error against a 64-bit solution is not larger in either precision.
 template <typename R>

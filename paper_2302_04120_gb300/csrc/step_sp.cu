@@ -21,11 +21,10 @@
 // digits of f_i ~ 1e3 kg m^-3; in FP64 it costs nothing because the deviation
 // form of every formula has the same operation count.
 //
-// MRT without matrices: [M]_dim = D [M] with D = diag(c^n), so the relaxation
-// is done on the lattice-scaled moments M f (integer combinations) with the
-// equilibrium and forcing moments divided by c^n, and [M]_dim^-1 is applied as
-// M^T diag(1/|row|^2) D^-1 -- the same arithmetic as the matrices of Sec. 3 /
-// App. A up to rounding order.
+// MRT without matrices: [M]_dim = D [M] with D = diag(c^n), so the operator of Sec. 3 / App. A
+// is that of the lattice-scaled moments; on half sums and half differences of opposite
+// populations it is a handful of products (sp_device.cuh), with factors folded on the host.
+// BGK is the same operator with all rates dt / tau.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
