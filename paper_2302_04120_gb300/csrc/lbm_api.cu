@@ -1043,10 +1043,13 @@ extern "C" void lbm_batch_destroy(lbm_batch_t b) {
 // one launch over all against single solves:
 //   calls of 48 steps (4 and 8: the same order): 20 MB 41 and 23, 30 MB 43 and 33, 42 MB 45 and
 //   45, 50 MB 47 and 54, 60 MB 48 and 56, 80 MB 49 and 60, 100 MB 50 and 54, 120 MB 48 and 52,
-//   140 MB 51 and 47, 180 MB 50 and 48, 300 MB 49 and 55 (by then with the build for large grids);
+//   140 MB 51 and 51, 180 MB 53 and 52, 220 MB 53 and 53, 300 MB 52 and 55;
 //   calls of 200 steps, which replay graphs (host calls hidden): 25 MB 45 and 42, 35 MB 46 and
 //   54, 42 MB 46 and 63, 60 MB 50 and 75, 100 MB 50 and 65, 140 MB 51 and 52, 180 MB 50 and 52,
 //   300 MB 49 and 58.
+// In uneven batches, where the shared launches are smaller, large channels alone gain more: 48
+// channels of 1 to 204 MB, 48 steps with initial fields and read-out, 29.0 ms with those of 129
+// to 240 MB in the shared launches, 28.2 without (30.6 one launch over all).
 // Sharing launches in groups that stay in L2 lost against one launch over all (48 channels of
 // 5 MB: 37 over all, 27 in groups of 60 MB, 34 of 90 MB; of 16 MB: 42, 26, 36).  The launches of
 // the others cost a few us per step that their nodes would not cost in the launch over all,
@@ -1060,8 +1063,7 @@ static bool batch_alone(const lbm_t h, int c) {
   if (h->p.precision == LBM_FP64 || h->launch_kind == LBM_LAUNCH_TMA) return false;
   const dim3 blk = step_launch(h).block;  // (a shape set by the caller may need too many rows of blocks)
   if ((h->p.ny + blk.y - 1) / blk.y > 65535) return false;
-  const double s = state_bytes(h);
-  return c ? s > 32e6 : (s > 55e6 && s < 129e6) || s > 240e6;
+  return state_bytes(h) > (c ? 32e6 : 45e6);
 }
 
 // Brings alone[] up to date with the channels' launches; whether it changed.
