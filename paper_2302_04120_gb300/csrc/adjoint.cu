@@ -304,7 +304,7 @@ __device__ __forceinline__ bool adj_frame_node(int nx, int ny, int f, int &i, in
 // Blocks of two warps: nothing is shared between warps (each adds its own dL/dnu partial,
 // summed in a fixed order), so no warp waits at a barrier.
 // Measured on 1024 x 128 (one launch, cold caches): FP64 129 -> 47 us (348 -> about 150 FP64
-// instructions per node), FP32 28 -> 15.7 us.
+// instructions per node), FP32 28 -> 15.2 us.
 constexpr int kAdjThreads = 64;
 template <typename S, typename R>
 __global__ void __launch_bounds__(kAdjThreads, sizeof(R) == 4 ? 16 : 8) k_adj_step(

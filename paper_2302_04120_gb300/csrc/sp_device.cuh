@@ -520,7 +520,7 @@ __device__ __forceinline__ void collide_bgk_T(const SpParams &P, const Macro<R> 
 // is exact, and of the rest population, what the source and the pairs leave.
 // T - T_in against the FP64 form, relative L2: 1024 x 128 channel with q = 1e6 W/m^3, 2000 steps
 // 1.8e-5 through S, 1.4e-6 this way (10000 steps: 5e-5, 3.5e-6); 700 x 96 without a source,
-// 10000 steps 5.7e-6, 1.3e-6.  Cost on 8192 x 4096: 0.9 % of the step.
+// 10000 steps 5.7e-6, 1.3e-6.  Cost: 0.6 % of the step on 8192 x 4096, 0.4 % on 2048 x 256.
 template <typename R>
 __device__ __forceinline__ void collide_mrt5(const SpParams &P, const Macro<R> &m, R g[5]) {
   const SpConst<R> &k = K<R>(P);
