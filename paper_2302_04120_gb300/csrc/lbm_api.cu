@@ -1271,7 +1271,7 @@ extern "C" lbm_status lbm_batch_step(lbm_batch_t b, long n) {
   if (n == 0) return LBM_OK;
   for (int k = 0; k < b->n; k++)  // the batched launch does not refresh a lagged qdot
     if (b->ch[k]->sink_conv != 0.0) return bfail(b, LBM_ERR_ARG, "channel %d has a lagged sink", k);
-  const bool changed = batch_split(b);
+  const bool changed = !recording(b->ch[0]) && batch_split(b);  // (new tile lists would end a caller's capture)
   lbm_status st = batch_tiles(b, b->bx, b->by, changed);
   if (st != LBM_OK) return st;
   int cur, pre;

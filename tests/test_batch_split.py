@@ -88,6 +88,35 @@ def test_tall_channel_with_a_launch_of_too_many_rows():
     b.close()
 
 
+def test_captured_call_after_a_launch_change():
+    """A channel's launch set just before the caller captures a call: the capture holds, and its
+    replay advances every channel as the call itself does."""
+    ws = [_w(nx, ny) for nx, ny in [(1100, 700), (1000, 512), (33, 7), (1060, 550)]]
+    st = torch.cuda.Stream()
+    out = []
+    for captured in (True, False):
+        b = lbm.Batch([w["params"] for w in ws], precision=1, stream=st.cuda_stream)
+        for ch, w in zip(b.channels, ws):
+            ch.apply_workload(w)
+        b.step(7)
+        b.step(4)  # (the tables are those of this call's buffers, which a capture cannot upload)
+        st.synchronize()
+        b.channels[1].set_launch(lbm.LBM_LAUNCH_TMA, 4, 2, 1)
+        if captured:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=st):
+                b.step(6)
+            with torch.cuda.stream(st):
+                graph.replay()
+        else:
+            b.step(6)
+        st.synchronize()
+        out.append([ch.moments() for ch in b.channels])
+        b.close()
+    for k, (a, r) in enumerate(zip(*out)):
+        _same(a, r, 17, k)
+
+
 def _shape(mb, k):
     nodes = mb * 1e6 / 112
     nx = int(round(math.sqrt(4 * nodes))) + k % 5
