@@ -510,6 +510,14 @@ __device__ __forceinline__ void collide_bgk_T(const SpParams &P, const Macro<R> 
   g[8] += p68 + o68;
 }
 
+// Adds x to the rest population; returns what its rounding left of x.
+template <typename R>
+__device__ __forceinline__ R rest_change(R &g0, R x) {
+  const R n = g0 + x, left = x - (n - g0);
+  g0 = n;
+  return left;
+}
+
 // Thermal MRT on D2Q5: moments (1, c_x, c_y, 5|c|^2 - 4c^2, c_x^2 - c_y^2), rates
 // (0, 1/tau_T, 1/tau_T, 1/dt, 1/dt), source Delta t (I - dt Lambda/2) M (w qdot).  The two
 // even moments at rate 1/dt take every even pair to w S, S = sum g + dt qdot.
@@ -517,10 +525,13 @@ __device__ __forceinline__ void collide_bgk_T(const SpParams &P, const Macro<R> 
 // In FP32 a source of one step is about a unit in the last place of sum g, or less: S rounded
 // loses or doubles it, the same way step after step at a node, and sum g drifts without a
 // source too.  So that form adds changes: of the pairs, w (S - a / 2 w) from a difference that
-// is exact, and of the rest population, what the source and the pairs leave.
+// is exact, of the rest population, what the source and the pairs leave, and what its own
+// rounding leaves of that goes to the axis pairs, whose odd parts keep their rounding from
+// repeating.
 // T - T_in against the FP64 form, relative L2: 1024 x 128 channel with q = 1e6 W/m^3, 2000 steps
-// 1.8e-5 through S, 1.4e-6 this way (10000 steps: 5e-5, 3.5e-6); 700 x 96 without a source,
-// 10000 steps 5.7e-6, 1.3e-6.  Cost: 0.6 % of the step on 8192 x 4096, 0.4 % on 2048 x 256.
+// 1.8e-5 through S, 1.4e-6 with changes, 9.6e-7 with the remainder (1e5 W/m^3, 50000 steps: 1.0e-5
+// with changes, 1.3e-6); 700 x 96 without a source, 10000 steps 5.7e-6 through S, 1.3e-6.
+// Cost: 0.4 % of the step on 8192 x 4096, 0.6 % on 2048 x 256.
 template <typename R>
 __device__ __forceinline__ void collide_mrt5(const SpParams &P, const Macro<R> &m, R g[5]) {
   const SpConst<R> &k = K<R>(P);
@@ -536,7 +547,9 @@ __device__ __forceinline__ void collide_mrt5(const SpParams &P, const Macro<R> &
     const R dS = P.qdot ? k.dt * m.qd : (R)0;
     px = w * (fma((R)-3, a13, m.sumg) + dS);
     py = w * (fma((R)-3, a24, m.sumg) + dS);
-    g[0] += dS - (R)2 * (px + py);
+    const R left = rest_change(g[0], dS - (R)2 * (px + py));
+    px += (R)0.25 * left;
+    py += (R)0.25 * left;
   }
   const R ex = off_eq(m, k.T0, d13, m.hx), ey = off_eq(m, k.T0, d24, m.hy);
   g[1] += px - k.hsT * ex;
@@ -565,23 +578,14 @@ __device__ __forceinline__ void collide_mrt9T(const SpParams &P, const Macro<R> 
     p68 = p36 - (R)0.5 * a68;
     g[0] = S - (R)4 * (p9 + p36);
   } else {
-    // (without a source w S rounded: its two weights' differences left sum g a drift of 2.5e-6
-    // of T - T_in after 10000 steps of a 500 x 50 half channel, this way 1e-6)
-    R dS = (R)0;
-    if (P.qdot) {
-      dS = k.dt * m.qd;
-      p13 = w4 * (fma((R)-4.5, a13, m.sumg) + dS);
-      p24 = w4 * (fma((R)-4.5, a24, m.sumg) + dS);
-      p57 = w8 * (fma((R)-18, a57, m.sumg) + dS);
-      p68 = w8 * (fma((R)-18, a68, m.sumg) + dS);
-    } else {
-      const R p9 = m.sumg * w4, p36 = m.sumg * w8;
-      p13 = p9 - (R)0.5 * a13;
-      p24 = p9 - (R)0.5 * a24;
-      p57 = p36 - (R)0.5 * a57;
-      p68 = p36 - (R)0.5 * a68;
-    }
-    g[0] += dS - (R)2 * ((p13 + p24) + (p57 + p68));
+    const R dS = P.qdot ? k.dt * m.qd : (R)0;
+    p13 = w4 * (fma((R)-4.5, a13, m.sumg) + dS);
+    p24 = w4 * (fma((R)-4.5, a24, m.sumg) + dS);
+    p57 = w8 * (fma((R)-18, a57, m.sumg) + dS);
+    p68 = w8 * (fma((R)-18, a68, m.sumg) + dS);
+    const R left = rest_change(g[0], dS - (R)2 * ((p13 + p24) + (p57 + p68)));
+    p13 += (R)0.25 * left;
+    p24 += (R)0.25 * left;
   }
   const R tx = d57 - d68, ty = d57 + d68;  // the diagonals' share of the first moment
   const R ex = off_eq(m, k.T0, d13 + tx, m.hx), ey = off_eq(m, k.T0, d24 + ty, m.hy);
